@@ -229,23 +229,90 @@ __global__ void __launch_bounds__(WG_CO * 27) k_wgrad3(const float* __restrict__
   if (col < WG_CO && cob + col < co_n) atomicAdd(&dW[((long long)(cob + col) * ci_n + ci) * 27 + tap], acc);
 }
 
-// db[c] += sum_{b, v} G[b][c][v]
-__global__ void __launch_bounds__(UT) k_bias_grad(const float* __restrict__ G, long long g_bs, int c_n, int B,
-                                                  long long n, float* __restrict__ db) {
-  const int c = blockIdx.x;
-  float acc = 0.f;
-  for (long long i = threadIdx.x; i < (long long)B * n; i += UT) {
-    const long long b = i / n, v = i % n;
-    acc += G[b * g_bs + (long long)c * n + v];
-  }
-  __shared__ float red[UT];
-  red[threadIdx.x] = acc;
+static cudaError_t wgrad3(const float* in, long long in_bs, int ci, const float* G, long long g_bs, int co, float* dW,
+                          int B, int nx, int ny, int nz, int bf, cudaStream_t st) {
+  const size_t smem = sizeof(float) * (3 * (WG_ROWS + 2) * (nx + 2) + WG_CO * WG_ROWS * nx);
+  cudaError_t e = cudaFuncSetAttribute(k_wgrad3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const long long chunks = (long long)B * nz * ((ny + WG_ROWS - 1) / WG_ROWS);
+  const long long rest = (long long)ci * ((co + WG_CO - 1) / WG_CO);
+  const long long want = std::max(1LL, std::min(chunks, (4LL * 152 + rest - 1) / rest));
+  const dim3 grid((unsigned)want, ci, (co + WG_CO - 1) / WG_CO);
+  k_wgrad3<<<grid, WG_CO * 27, smem, st>>>(in, in_bs, ci, G, g_bs, co, dW, B, nx, ny, nz, bf);
+  return cudaGetLastError();
+}
+
+// Sum over the CTA's threads of v, valid in thread 0 (FP32 within warps, FP32 across them).
+__device__ __forceinline__ float block_sum(float v) {
+  __shared__ float red[UT / 32];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
-  for (int o = UT / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float s = 0.f;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < UT / 32; ++w) s += red[w];
+  return s;
+}
+
+// Grid of the per-channel reductions below: RC_PER float4 (or values) per thread along a
+// channel plane in x, channels in y, samples in z.  A one-CTA-per-channel reduction leaves
+// 120 to 136 of 152 SMs idle at 16 to 32 channels (3.1 ms for a 0.2 GB tensor at
+// 24 x 64x64x32); here every CTA sums one chunk of a plane and adds it with one atomic.
+constexpr int RC_PER = 4;
+static dim3 chan_grid(long long n, int C, int B) {
+  const long long units = n % 4 == 0 ? n / 4 : n;
+  return dim3((unsigned)((units + UT * RC_PER - 1) / (UT * RC_PER)), C, std::min(B, 65535));
+}
+
+// g <- g * (y > 0) for a ReLU output y (MASK; sample strides allow concat views) and
+// db[c] += sum_{b, v} g[b][c][v], in one pass.
+template <bool MASK, bool VEC>
+__global__ void __launch_bounds__(UT) k_relu_bias_grad(float* __restrict__ g, long long g_bs,
+                                                       const float* __restrict__ y, long long y_bs, int B,
+                                                       long long n, float* __restrict__ db) {
+  const int c = blockIdx.y;
+  const long long units = VEC ? n / 4 : n;
+  const long long u0 = (long long)blockIdx.x * (UT * RC_PER) + threadIdx.x;
+  float acc = 0.f;
+  for (int b = blockIdx.z; b < B; b += gridDim.z) {
+    float* gp = g + b * g_bs + (long long)c * n;
+    const float* yp = MASK ? y + b * y_bs + (long long)c * n : nullptr;
+#pragma unroll
+    for (int k = 0; k < RC_PER; ++k) {
+      const long long u = u0 + k * UT;
+      if (u >= units) continue;
+      if constexpr (VEC) {
+        float4 v = reinterpret_cast<const float4*>(gp)[u];
+        if constexpr (MASK) {
+          const float4 m = reinterpret_cast<const float4*>(yp)[u];
+          v = make_float4(m.x > 0.f ? v.x : 0.f, m.y > 0.f ? v.y : 0.f, m.z > 0.f ? v.z : 0.f, m.w > 0.f ? v.w : 0.f);
+          reinterpret_cast<float4*>(gp)[u] = v;
+        }
+        acc += (v.x + v.y) + (v.z + v.w);
+      } else {
+        float v = gp[u];
+        if constexpr (MASK) {
+          v = yp[u] > 0.f ? v : 0.f;
+          gp[u] = v;
+        }
+        acc += v;
+      }
+    }
   }
-  if (threadIdx.x == 0) db[c] += red[0];
+  const float s = block_sum(acc);
+  if (threadIdx.x == 0) atomicAdd(&db[c], s);
+}
+
+template <bool MASK>
+static cudaError_t relu_bias_grad(float* g, long long g_bs, const float* y, long long y_bs, int C, int B, long long n,
+                                  float* db, cudaStream_t st) {
+  if (n % 4 == 0)
+    k_relu_bias_grad<MASK, true><<<chan_grid(n, C, B), UT, 0, st>>>(g, g_bs, y, y_bs, B, n, db);
+  else
+    k_relu_bias_grad<MASK, false><<<chan_grid(n, C, B), UT, 0, st>>>(g, g_bs, y, y_bs, B, n, db);
+  return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------- pooling, transposed conv, 1x1 conv
@@ -331,34 +398,74 @@ __global__ void k_tconv_dgrad(const float* __restrict__ dout, long long dout_bs,
   }
 }
 
-// dW[ci][co][d] += sum_{b, v} in[b][ci][v] dout[b][co][2v + d]: one CTA per (ci, co).
+// dW[ci][co][d] += sum_{b, v} in[b][ci][v] dout[b][co][2v + d].  A CTA takes 16 input and 4
+// output channels (16 x 4 x 8 sums, two per thread: d pairs of one (ci, co)) and a share of the
+// 64-voxel runs of (sample, z, y) rows; each run's inputs and children are staged once in
+// shared memory, so global memory is read once per channel block instead of once per
+// (ci, co) pair.  FP32 sums, one atomic per sum and CTA.
+constexpr int TW_CI = 16, TW_CO = 4, TW_V = 64;
 __global__ void __launch_bounds__(UT) k_tconv_wgrad(const float* __restrict__ in, int ci_n,
                                                     const float* __restrict__ dout, long long dout_bs, int co_n,
                                                     float* __restrict__ dW, int B, int nx, int ny, int nz, int bf) {
-  const int ci = blockIdx.x, co = blockIdx.y;
-  const long long n = (long long)nx * ny * nz, in_n = n / 8;
-  const int ix = nx / 2, iy = ny / 2;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (long long i = threadIdx.x; i < (long long)B * in_n; i += UT) {
-    const long long b = i / in_n, v = i % in_n;
-    const int x = (int)(v % ix), y = (int)((v / ix) % iy), z = (int)(v / ((long long)ix * iy));
-    const float xv = opr(in[(b * ci_n + ci) * in_n + v], bf);
-    const float* g = dout + b * dout_bs + (long long)co * n;
-#pragma unroll
-    for (int d = 0; d < 8; ++d)
-      acc[d] = fmaf(xv, opr(g[(long long)(2 * z + (d >> 2)) * nx * ny + (long long)(2 * y + ((d >> 1) & 1)) * nx + 2 * x + (d & 1)], bf),
-                    acc[d]);
-  }
-  __shared__ float red[8][UT];
-#pragma unroll
-  for (int d = 0; d < 8; ++d) red[d][threadIdx.x] = acc[d];
-  __syncthreads();
-  for (int o = UT / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int d = 0; d < 8; ++d) red[d][threadIdx.x] += red[d][threadIdx.x + o];
+  __shared__ float s_x[TW_CI][TW_V + 1];
+  __shared__ __align__(16) float s_g[TW_CO * 4][2 * TW_V + 2];   // rows (co, dz, dy) of 2 TW_V children
+  const int ix = nx / 2, iy = ny / 2, iz = nz / 2;
+  const long long n = (long long)nx * ny * nz, in_n = n / 8, iplane = (long long)ix * iy;
+  const int ci0 = blockIdx.y * TW_CI, co0 = blockIdx.z * TW_CO;
+  const int runs_x = (ix + TW_V - 1) / TW_V;
+  const long long runs = (long long)B * iz * iy * runs_x;
+  const int ci = threadIdx.x / 16, co = (threadIdx.x / 4) % 4, zy = threadIdx.x % 4;
+  float a0 = 0.f, a1 = 0.f;
+  for (long long r = blockIdx.x; r < runs; r += gridDim.x) {
+    const int x0 = (int)(r % runs_x) * TW_V;
+    long long t = r / runs_x;
+    const int y = (int)(t % iy);
+    t /= iy;
+    const int z = (int)(t % iz);
+    const long long b = t / iz;
+    const int w = min(TW_V, ix - x0);
     __syncthreads();
+    for (int e = threadIdx.x; e < TW_CI * TW_V; e += UT) {
+      const int c = e / TW_V, x = e % TW_V;
+      s_x[c][x] = ci0 + c < ci_n && x < w
+                      ? opr(__ldg(&in[(b * ci_n + ci0 + c) * in_n + z * iplane + (long long)y * ix + x0 + x]), bf)
+                      : 0.f;
+    }
+    for (int e = threadIdx.x; e < TW_CO * 4 * 2 * TW_V; e += UT) {
+      const int x = e % (2 * TW_V), row = e / (2 * TW_V), c = row / 4, d = row % 4;
+      s_g[row][x] = co0 + c < co_n && x < 2 * w
+                        ? opr(__ldg(&dout[b * dout_bs + (long long)(co0 + c) * n + (long long)(2 * z + (d >> 1)) * nx * ny +
+                                          (long long)(2 * y + (d & 1)) * nx + 2 * x0 + x]), bf)
+                        : 0.f;
+    }
+    __syncthreads();
+    const float* gp = s_g[co * 4 + zy];
+    const float* xp = s_x[ci];
+    float r0 = 0.f, r1 = 0.f;   // a run's sums apart: short FP32 chains
+#pragma unroll 8
+    for (int x = 0; x < TW_V; ++x) {
+      const float xv = xp[x];
+      const float2 g = *reinterpret_cast<const float2*>(gp + 2 * x);
+      r0 = fmaf(xv, g.x, r0);
+      r1 = fmaf(xv, g.y, r1);
+    }
+    a0 += r0;
+    a1 += r1;
   }
-  if (threadIdx.x < 8) dW[((long long)ci * co_n + co) * 8 + threadIdx.x] += red[threadIdx.x][0];
+  if (ci0 + ci < ci_n && co0 + co < co_n) {
+    float* d = &dW[((long long)(ci0 + ci) * co_n + co0 + co) * 8 + 2 * zy];
+    atomicAdd(d, a0);
+    atomicAdd(d + 1, a1);
+  }
+}
+
+static cudaError_t tconv_wgrad(const float* in, int ci, const float* dout, long long dout_bs, int co, float* dW, int B,
+                               int nx, int ny, int nz, int bf, cudaStream_t st) {
+  const int bi = (ci + TW_CI - 1) / TW_CI, bo = (co + TW_CO - 1) / TW_CO;
+  const long long runs = (long long)B * (nz / 2) * (ny / 2) * ((nx / 2 + TW_V - 1) / TW_V);
+  const long long per = std::max(1, 152 * 8 / (bi * bo));
+  k_tconv_wgrad<<<dim3((unsigned)std::min(runs, per), bi, bo), UT, 0, st>>>(in, ci, dout, dout_bs, co, dW, B, nx, ny, nz, bf);
+  return cudaGetLastError();
 }
 
 // 1x1x1 conv to one channel: out[b][v] = bias + sum_c W[c] in[b][c][v]
@@ -371,45 +478,50 @@ __global__ void k_conv1_fwd(const float* __restrict__ in, int c_n, const float* 
     out[i] = acc;
   }
 }
-// din[b][c][v] = W[c] dout[b][v]
-__global__ void k_conv1_dgrad(const float* __restrict__ dout, int c_n, const float* __restrict__ W,
-                              float* __restrict__ din, int B, long long n, int bf) {
-  for (long long i = (long long)blockIdx.x * UT + threadIdx.x; i < (long long)B * c_n * n; i += (long long)gridDim.x * UT) {
-    const long long v = i % n, bc = i / n;
-    const int c = (int)(bc % c_n);
-    const long long b = bc / c_n;
-    din[i] = opr(W[c], bf) * opr(dout[b * n + v], bf);
+// Backward of the 1x1x1 conv and of the ReLU before it, in one pass over the input `in` (the
+// ReLU output): din[b][c][v] = W[c] dout[b][v] where in > 0, else 0; dW[c] += sum in dout;
+// db += sum dout (once, by channel 0's CTAs); dbprev[c] += sum din (the bias of the layer
+// that made `in`).
+template <bool VEC>
+__global__ void __launch_bounds__(UT) k_conv1_bwd(const float* __restrict__ in, int c_n, const float* __restrict__ dout,
+                                                  const float* __restrict__ W, float* __restrict__ din,
+                                                  float* __restrict__ dW, float* __restrict__ db,
+                                                  float* __restrict__ dbprev, int B, long long n, int bf) {
+  const int c = blockIdx.y;
+  const long long units = VEC ? n / 4 : n;
+  const long long u0 = (long long)blockIdx.x * (UT * RC_PER) + threadIdx.x;
+  const float w = opr(__ldg(&W[c]), bf);
+  float sw = 0.f, sb = 0.f, sp = 0.f;
+  for (int b = blockIdx.z; b < B; b += gridDim.z) {
+    const float* ip = in + ((long long)b * c_n + c) * n;
+    float* op = din + ((long long)b * c_n + c) * n;
+    const float* gp = dout + (long long)b * n;
+    auto one = [&](float x, float g) {
+      const float gr = opr(g, bf), d = x > 0.f ? w * gr : 0.f;
+      sw = fmaf(opr(x, bf), gr, sw);
+      sb += g;
+      sp += d;
+      return d;
+    };
+#pragma unroll
+    for (int k = 0; k < RC_PER; ++k) {
+      const long long u = u0 + k * UT;
+      if (u >= units) continue;
+      if constexpr (VEC) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(ip) + u), g = __ldg(reinterpret_cast<const float4*>(gp) + u);
+        reinterpret_cast<float4*>(op)[u] = make_float4(one(x.x, g.x), one(x.y, g.y), one(x.z, g.z), one(x.w, g.w));
+      } else {
+        op[u] = one(__ldg(ip + u), __ldg(gp + u));
+      }
+    }
   }
-}
-// dW[c] += sum in[b][c][v] dout[b][v] (one CTA per channel; c == c_n: the bias)
-__global__ void __launch_bounds__(UT) k_conv1_wgrad(const float* __restrict__ in, int c_n,
-                                                    const float* __restrict__ dout, float* __restrict__ dW,
-                                                    float* __restrict__ db, int B, long long n, int bf) {
-  const int c = blockIdx.x;
-  float acc = 0.f;
-  for (long long i = threadIdx.x; i < (long long)B * n; i += UT) {
-    const long long b = i / n, v = i % n;
-    acc += (c < c_n ? opr(in[(b * c_n + c) * n + v], bf) * opr(dout[i], bf) : dout[i]);
-  }
-  __shared__ float red[UT];
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int o = UT / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
+  sw = block_sum(sw);
+  sb = block_sum(sb);
+  sp = block_sum(sp);
   if (threadIdx.x == 0) {
-    if (c < c_n) dW[c] += red[0];
-    else db[0] += red[0];
-  }
-}
-
-// g <- g * (y > 0) for a ReLU output y (sample strides allow concat views)
-__global__ void k_relu_bwd(float* __restrict__ g, long long g_bs, const float* __restrict__ y, long long y_bs,
-                           int C, int B, long long n) {
-  for (long long i = (long long)blockIdx.x * UT + threadIdx.x; i < (long long)B * C * n; i += (long long)gridDim.x * UT) {
-    const long long b = i / ((long long)C * n), r = i % ((long long)C * n);
-    if (!(y[b * y_bs + r] > 0.f)) g[b * g_bs + r] = 0.f;
+    atomicAdd(&dW[c], sw);
+    atomicAdd(&dbprev[c], sp);
+    if (c == 0) atomicAdd(db, sb);
   }
 }
 
@@ -741,27 +853,17 @@ extern "C" clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float*
 }
 
 // conv3 backward for layer li: input `in` (ci channels, sample stride in_bs), output gradient
-// `g` (co channels, stride g_bs); writes din (if non-NULL) and accumulates dW, db.
+// `g` (co channels, stride g_bs); writes din (if non-NULL) and accumulates dW.
 static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long in_bs, const float* g, long long g_bs,
                               float* din, long long din_bs, int B, int nx, int ny, int nz, cudaStream_t st) {
   const Layer& L = u->layers[li];
   const bool bf = u->bf != 0;
-  const long long n = (long long)nx * ny * nz;
   if (din) {
     k_flip<<<grid_for((long long)L.nw), UT, 0, st>>>(u->p + L.w, u->flip, L.ci, L.co);
     U_TRY(cudaGetLastError());
     U_TRY(conv3(bf, g, g_bs, L.co, din, din_bs, L.ci, u->flip, nullptr, false, B, nx, ny, nz, st, u->ctx()));
   }
-  const size_t smem = sizeof(float) * (3 * (WG_ROWS + 2) * (nx + 2) + WG_CO * WG_ROWS * nx);
-  U_TRY(cudaFuncSetAttribute(k_wgrad3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const long long chunks = (long long)B * nz * ((ny + WG_ROWS - 1) / WG_ROWS);
-  const long long rest = (long long)L.ci * ((L.co + WG_CO - 1) / WG_CO);
-  const long long want = std::max(1LL, std::min(chunks, (4LL * 152 + rest - 1) / rest));
-  dim3 grid((unsigned)want, L.ci, (L.co + WG_CO - 1) / WG_CO);
-  k_wgrad3<<<grid, WG_CO * 27, smem, st>>>(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->bf);
-  U_TRY(cudaGetLastError());
-  k_bias_grad<<<L.co, UT, 0, st>>>(g, g_bs, L.co, B, n, u->g + L.b);
-  U_TRY(cudaGetLastError());
+  U_TRY(wgrad3(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->bf, st));
   return CLAMP_OK;
 }
 
@@ -791,62 +893,60 @@ extern "C" clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const
     U_TRY(cudaGetLastError());
   }
   auto W = [&](int i) { return u->p + u->layers[i].w; };
-  // output 1x1 conv
-  k_conv1_dgrad<<<grid_for(B * c1 * n1), UT, 0, st>>>(a.gout, c1, W(12), a.gd1b, B, n1, bf);
-  k_conv1_wgrad<<<c1 + 1, UT, 0, st>>>(a.d1b, c1, a.gout, u->g + u->layers[12].w, u->g + u->layers[12].b, B, n1, bf);
+  auto dB = [&](int i) { return u->g + u->layers[i].b; };
+  // output 1x1 conv, the ReLU before it and that layer's bias
+  (n1 % 4 == 0 ? k_conv1_bwd<true> : k_conv1_bwd<false>)<<<chan_grid(n1, c1, B), UT, 0, st>>>(
+      a.d1b, c1, a.gout, W(12), a.gd1b, u->g + u->layers[12].w, dB(12), dB(11), B, n1, bf);
   U_TRY(cudaGetLastError());
   // decoder level 1
-  k_relu_bwd<<<grid_for(B * c1 * n1), UT, 0, st>>>(a.gd1b, c1 * n1, a.d1b, c1 * n1, c1, B, n1);
   s = conv3_bwd(u, 11, a.d1a, c1 * n1, a.gd1b, c1 * n1, a.gd1a, c1 * n1, B, nx, ny, nz, st);
   if (s != CLAMP_OK) return s;
-  k_relu_bwd<<<grid_for(B * c1 * n1), UT, 0, st>>>(a.gd1a, c1 * n1, a.d1a, c1 * n1, c1, B, n1);
+  U_TRY(relu_bias_grad<true>(a.gd1a, c1 * n1, a.d1a, c1 * n1, c1, B, n1, dB(10), st));
   s = conv3_bwd(u, 10, a.cat1, 2 * c1 * n1, a.gd1a, c1 * n1, a.gcat1, 2 * c1 * n1, B, nx, ny, nz, st);
   if (s != CLAMP_OK) return s;
   // transposed conv up1: u1 = cat1[:, :c1] from d2b
   k_tconv_dgrad<<<grid_for(B * c2 * n2), UT, 0, st>>>(a.gcat1, 2 * c1 * n1, c1, a.gd2b, c2, W(9), B, nx, ny, nz, bf);
-  k_tconv_wgrad<<<dim3(c2, c1), UT, 0, st>>>(a.d2b, c2, a.gcat1, 2 * c1 * n1, c1, u->g + u->layers[9].w, B, nx, ny, nz, bf);
-  k_bias_grad<<<c1, UT, 0, st>>>(a.gcat1, 2 * c1 * n1, c1, B, n1, u->g + u->layers[9].b);
   U_TRY(cudaGetLastError());
+  U_TRY(tconv_wgrad(a.d2b, c2, a.gcat1, 2 * c1 * n1, c1, u->g + u->layers[9].w, B, nx, ny, nz, bf, st));
+  U_TRY(relu_bias_grad<false>(a.gcat1, 2 * c1 * n1, nullptr, 0, c1, B, n1, dB(9), st));
   // decoder level 2
-  k_relu_bwd<<<grid_for(B * c2 * n2), UT, 0, st>>>(a.gd2b, c2 * n2, a.d2b, c2 * n2, c2, B, n2);
+  U_TRY(relu_bias_grad<true>(a.gd2b, c2 * n2, a.d2b, c2 * n2, c2, B, n2, dB(8), st));
   s = conv3_bwd(u, 8, a.d2a, c2 * n2, a.gd2b, c2 * n2, a.gd2a, c2 * n2, B, hx, hy, hz, st);
   if (s != CLAMP_OK) return s;
-  k_relu_bwd<<<grid_for(B * c2 * n2), UT, 0, st>>>(a.gd2a, c2 * n2, a.d2a, c2 * n2, c2, B, n2);
+  U_TRY(relu_bias_grad<true>(a.gd2a, c2 * n2, a.d2a, c2 * n2, c2, B, n2, dB(7), st));
   s = conv3_bwd(u, 7, a.cat2, 2 * c2 * n2, a.gd2a, c2 * n2, a.gcat2, 2 * c2 * n2, B, hx, hy, hz, st);
   if (s != CLAMP_OK) return s;
   // transposed conv up2: u2 = cat2[:, :c2] from btb
   k_tconv_dgrad<<<grid_for(B * c3 * n3), UT, 0, st>>>(a.gcat2, 2 * c2 * n2, c2, a.gbtb, c3, W(6), B, hx, hy, hz, bf);
-  k_tconv_wgrad<<<dim3(c3, c2), UT, 0, st>>>(a.btb, c3, a.gcat2, 2 * c2 * n2, c2, u->g + u->layers[6].w, B, hx, hy, hz, bf);
-  k_bias_grad<<<c2, UT, 0, st>>>(a.gcat2, 2 * c2 * n2, c2, B, n2, u->g + u->layers[6].b);
   U_TRY(cudaGetLastError());
+  U_TRY(tconv_wgrad(a.btb, c3, a.gcat2, 2 * c2 * n2, c2, u->g + u->layers[6].w, B, hx, hy, hz, bf, st));
+  U_TRY(relu_bias_grad<false>(a.gcat2, 2 * c2 * n2, nullptr, 0, c2, B, n2, dB(6), st));
   // bottleneck
-  k_relu_bwd<<<grid_for(B * c3 * n3), UT, 0, st>>>(a.gbtb, c3 * n3, a.btb, c3 * n3, c3, B, n3);
+  U_TRY(relu_bias_grad<true>(a.gbtb, c3 * n3, a.btb, c3 * n3, c3, B, n3, dB(5), st));
   s = conv3_bwd(u, 5, a.bta, c3 * n3, a.gbtb, c3 * n3, a.gbta, c3 * n3, B, qx, qy, qz, st);
   if (s != CLAMP_OK) return s;
-  k_relu_bwd<<<grid_for(B * c3 * n3), UT, 0, st>>>(a.gbta, c3 * n3, a.bta, c3 * n3, c3, B, n3);
+  U_TRY(relu_bias_grad<true>(a.gbta, c3 * n3, a.bta, c3 * n3, c3, B, n3, dB(4), st));
   s = conv3_bwd(u, 4, a.p2, c2 * n3, a.gbta, c3 * n3, a.gp2, c2 * n3, B, qx, qy, qz, st);
   if (s != CLAMP_OK) return s;
   // pool 2 into the skip s2 = cat2[:, c2:] (its gradient already holds the concat path)
   k_pool_bwd<<<grid_for(B * c2 * n3), UT, 0, st>>>(a.gp2, a.arg2, a.gcat2 + c2 * n2, 2 * c2 * n2, c2, B, hx, hy, hz);
   U_TRY(cudaGetLastError());
   // encoder level 2
-  k_relu_bwd<<<grid_for(B * c2 * n2), UT, 0, st>>>(a.gcat2 + c2 * n2, 2 * c2 * n2, a.cat2 + c2 * n2, 2 * c2 * n2, c2, B, n2);
+  U_TRY(relu_bias_grad<true>(a.gcat2 + c2 * n2, 2 * c2 * n2, a.cat2 + c2 * n2, 2 * c2 * n2, c2, B, n2, dB(3), st));
   s = conv3_bwd(u, 3, a.e2a, c2 * n2, a.gcat2 + c2 * n2, 2 * c2 * n2, a.ge2a, c2 * n2, B, hx, hy, hz, st);
   if (s != CLAMP_OK) return s;
-  k_relu_bwd<<<grid_for(B * c2 * n2), UT, 0, st>>>(a.ge2a, c2 * n2, a.e2a, c2 * n2, c2, B, n2);
+  U_TRY(relu_bias_grad<true>(a.ge2a, c2 * n2, a.e2a, c2 * n2, c2, B, n2, dB(2), st));
   s = conv3_bwd(u, 2, a.p1, c1 * n2, a.ge2a, c2 * n2, a.gp1, c1 * n2, B, hx, hy, hz, st);
   if (s != CLAMP_OK) return s;
   // pool 1 into the skip s1 = cat1[:, c1:]
   k_pool_bwd<<<grid_for(B * c1 * n2), UT, 0, st>>>(a.gp1, a.arg1, a.gcat1 + c1 * n1, 2 * c1 * n1, c1, B, nx, ny, nz);
   U_TRY(cudaGetLastError());
   // encoder level 1
-  k_relu_bwd<<<grid_for(B * c1 * n1), UT, 0, st>>>(a.gcat1 + c1 * n1, 2 * c1 * n1, a.cat1 + c1 * n1, 2 * c1 * n1, c1, B, n1);
+  U_TRY(relu_bias_grad<true>(a.gcat1 + c1 * n1, 2 * c1 * n1, a.cat1 + c1 * n1, 2 * c1 * n1, c1, B, n1, dB(1), st));
   s = conv3_bwd(u, 1, a.e1a, c1 * n1, a.gcat1 + c1 * n1, 2 * c1 * n1, a.ge1a, c1 * n1, B, nx, ny, nz, st);
   if (s != CLAMP_OK) return s;
-  k_relu_bwd<<<grid_for(B * c1 * n1), UT, 0, st>>>(a.ge1a, c1 * n1, a.e1a, c1 * n1, c1, B, n1);
-  s = conv3_bwd(u, 0, x, n1, a.ge1a, c1 * n1, nullptr, 0, B, nx, ny, nz, st);
-  if (s != CLAMP_OK) return s;
-  return CLAMP_OK;
+  U_TRY(relu_bias_grad<true>(a.ge1a, c1 * n1, a.e1a, c1 * n1, c1, B, n1, dB(0), st));
+  return conv3_bwd(u, 0, x, n1, a.ge1a, c1 * n1, nullptr, 0, B, nx, ny, nz, st);
 }
 
 extern "C" clamp_status clamp_unet_adam(clamp_unet* u, float lr, float beta1, float beta2, float eps, int32_t t,
