@@ -182,63 +182,225 @@ __global__ void k_flip(const float* __restrict__ W, float* __restrict__ Wf, int 
   }
 }
 
-// dW[co][ci][tap] += sum_{b, v} G[b][co][v] in[b][ci][v + tap], for one input channel ci and 16
-// output channels per CTA; CTAs stride over (sample, plane, 4-row) chunks; atomics combine them.
-constexpr int WG_CO = 16, WG_ROWS = 4;
-__global__ void __launch_bounds__(WG_CO * 27) k_wgrad3(const float* __restrict__ in, long long in_bs, int ci_n,
-                                                       const float* __restrict__ G, long long g_bs, int co_n,
-                                                       float* __restrict__ dW, int B, int nx, int ny, int nz, int bf) {
-  extern __shared__ float sm[];
-  const int IXH = nx + 2, halo = 3 * (WG_ROWS + 2) * IXH, vox = WG_ROWS * nx;
-  float* s_x = sm;              // [3][ROWS+2][nx+2]
-  float* s_g = sm + halo;       // [WG_CO][ROWS][nx]
-  const int ci = blockIdx.y, cob = blockIdx.z * WG_CO;
-  const int t = threadIdx.x, col = t / 27, tap = t % 27;
-  const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
+// dW[co][ci][tap] += sum_{b, v} G[b][co][v] in[b][ci][v + tap] on the CUDA cores: one FP32 chain
+// per (co, ci, tap) and share of the volume, in voxel order over the share's (sample, plane,
+// 4-row) chunks; atomics combine the shares.  A CTA takes CIC input channels and COB output
+// channels: a consumer warp per input channel, lane = (output channel, half of the taps), 14
+// chains per lane in registers.  The x taps come from a window that slides along the row,
+// so four voxels cost six 16-byte shared loads and 56 FMAs, where a thread per chain paid
+// two loads per FMA (16 -> 16 at 24 x 64x64x32: 12.3 -> 1.46 ms).  Producer warps stage the next
+// chunk meanwhile (two buffers where they fit).  Bound by the issue of one consumer warp per
+// scheduler: 56 FMAs of about 90 instructions per four voxels, FMA pipe 47 % busy.
+constexpr int WG_CO = 16, WG_ROWS = 4, WG_NT = 512;
+__host__ __device__ constexpr int wg_pitch(int nx) { return (nx + 3) / 4 * 4 + 8; }   // 4 zeros left, >= 4 right
+__host__ __device__ constexpr int wg_gstride(int nx) { return (WG_ROWS * ((nx + 3) / 4 * 4) + 31) / 32 * 32 + 4; }
+static size_t wg_buf_floats(int cic, int cob, int nx) {
+  return (size_t)3 * (WG_ROWS + 2) * cic * wg_pitch(nx) + (size_t)cob * wg_gstride(nx) + 4;
+}
+
+template <int CIC, int COB, bool VEC>
+__global__ void __launch_bounds__(WG_NT) k_wgrad3(const float* __restrict__ in, long long in_bs, int ci_n,
+                                                  const float* __restrict__ G, long long g_bs, int co_n,
+                                                  float* __restrict__ dW, int B, int nx, int ny, int nz, int bf,
+                                                  int nbuf) {
+  extern __shared__ __align__(16) float wg_sm[];
+  constexpr int XR = 3 * (WG_ROWS + 2);   // X rows per channel: [dz][row]
+  const int nq = (nx + 3) / 4, pitch = wg_pitch(nx), gs = wg_gstride(nx);
+  const int buf_floats = XR * CIC * pitch + COB * gs + 4;   // 4: the look-ahead's last read
+  const int ci0 = blockIdx.y * CIC, cob = blockIdx.z * COB;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long plane = (long long)nx * ny, n = plane * nz;
   const int row_blocks = (ny + WG_ROWS - 1) / WG_ROWS;
   const long long chunks = (long long)B * nz * row_blocks;
-  float acc = 0.f;
-  for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
-    const int rb = (int)(ch % row_blocks), z = (int)((ch / row_blocks) % nz), b = (int)(ch / ((long long)row_blocks * nz));
-    const int y0 = rb * WG_ROWS;
-    __syncthreads();
-    for (int e = t; e < halo; e += blockDim.x) {
-      const int xi = e % IXH, yi = (e / IXH) % (WG_ROWS + 2), zi = e / (IXH * (WG_ROWS + 2));
-      const int gx = xi - 1, gy = y0 + yi - 1, gz = z + zi - 1;
-      float v = 0.f;
-      if (gx >= 0 && gx < nx && gy >= 0 && gy < ny && gz >= 0 && gz < nz)
-        v = in[(long long)b * in_bs + (long long)ci * n + (long long)gz * plane + (long long)gy * nx + gx];
-      s_x[e] = opr(v, bf);
-    }
-    for (int e = t; e < WG_CO * vox; e += blockDim.x) {
-      const int o = e / vox, r = (e % vox) / nx, x = e % nx;
-      const int co = cob + o, gy = y0 + r;
-      s_g[e] = (co < co_n && gy < ny) ? opr(G[(long long)b * g_bs + (long long)co * n + (long long)z * plane + (long long)gy * nx + x], bf) : 0.f;
-    }
-    __syncthreads();
-    if (col < WG_CO) {
-      const float* g = s_g + col * vox;
-      for (int r = 0; r < WG_ROWS; ++r) {
-        const float* xr = s_x + (dz * (WG_ROWS + 2) + r + dy) * IXH + dx;
-        const float* gr = g + r * nx;
-        for (int x = 0; x < nx; ++x) acc = fmaf(gr[x], xr[x], acc);
-      }
+  for (int e = threadIdx.x; e < nbuf * buf_floats; e += (int)blockDim.x) wg_sm[e] = 0.f;   // halo columns stay zero
+  __syncthreads();
+
+  // Where each staged row comes from and goes: {channel, offset of the row from the chunk's first
+  // voxel, offset in the buffer, what must lie inside the volume: bits of X rows 0..5, planes
+  // 8..10, G rows 16..19; bit 31: no such channel}.
+  constexpr int ROWS = XR * CIC + COB * WG_ROWS, UN = 6;
+  __shared__ int4 s_row[ROWS];
+  for (int r = threadIdx.x; r < ROWS; r += (int)blockDim.x) {
+    const int f = r - XR * CIC;
+    if (f < 0) {   // X row [channel][dz][row]
+      const int row = r % (WG_ROWS + 2), dz = (r / (WG_ROWS + 2)) % 3, c = r / XR;
+      s_row[r] = make_int4(c, (int)((dz - 1) * plane) + (row - 1) * nx, r * pitch + 4,
+                           ci0 + c < ci_n ? (1 << row) | (1 << (8 + dz)) : (int)0x80000000);
+    } else {       // G row [output channel][row]
+      const int o = f / WG_ROWS, row = f % WG_ROWS;
+      s_row[r] = make_int4(o, row * nx, XR * CIC * pitch + o * gs + row * nq * 4,
+                           cob + o < co_n ? 1 << (16 + row) : (int)0x80000000);
     }
   }
-  if (col < WG_CO && cob + col < co_n) atomicAdd(&dW[((long long)(cob + col) * ci_n + ci) * 27 + tap], acc);
+  __syncthreads();
+
+  // Threads 0 <= t < nt stage chunk ch into buffer `to`: groups of 2^lq threads along a row's
+  // quads, six rows' loads in flight per thread.
+  const int lq = nq > 16 ? 5 : nq > 8 ? 4 : nq > 4 ? 3 : 2;
+  auto stage = [&](long long ch, float* to, int t, int nt) {
+    const int rb = (int)(ch % row_blocks), z = (int)((ch / row_blocks) % nz), b = (int)(ch / ((long long)row_blocks * nz));
+    const int y0 = rb * WG_ROWS, q0 = t & ((1 << lq) - 1), rstep = nt >> lq;
+    const long long v0 = z * plane + (long long)y0 * nx;
+    const float* xb = in + b * in_bs + (long long)ci0 * n + v0;
+    const float* gb = G + b * g_bs + (long long)cob * n + v0;
+    int inside = (z > 0 ? 1 << 8 : 0) | 1 << 9 | (z + 1 < nz ? 1 << 10 : 0);
+#pragma unroll
+    for (int r = 0; r < WG_ROWS + 2; ++r) {
+      const int gy = y0 + r - 1;
+      if (gy >= 0 && gy < ny) inside |= 1 << r;
+      if (r < WG_ROWS && y0 + r < ny) inside |= 1 << (16 + r);
+    }
+    for (int q = q0; q < nq; q += 1 << lq) {
+      for (int r0 = t >> lq; r0 < ROWS; r0 += UN * rstep) {
+        float4 v[UN];
+        int dst[UN];
+#pragma unroll
+        for (int k = 0; k < UN; ++k) {
+          const int r = r0 + k * rstep;
+          v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          dst[k] = -1;
+          if (r >= ROWS) continue;
+          const int4 e = s_row[r];
+          dst[k] = e.z;
+          if ((e.w & inside) != e.w) continue;
+          const float* src = (r < XR * CIC ? xb : gb) + e.x * n + e.y;
+          if constexpr (VEC) {
+            v[k] = __ldg(reinterpret_cast<const float4*>(src) + q);
+          } else {
+            v[k].x = __ldg(src + 4 * q);
+            if (4 * q + 1 < nx) v[k].y = __ldg(src + 4 * q + 1);
+            if (4 * q + 2 < nx) v[k].z = __ldg(src + 4 * q + 2);
+            if (4 * q + 3 < nx) v[k].w = __ldg(src + 4 * q + 3);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < UN; ++k)
+          if (dst[k] >= 0)
+            reinterpret_cast<float4*>(to + dst[k])[q] =
+                make_float4(opr(v[k].x, bf), opr(v[k].y, bf), opr(v[k].z, bf), opr(v[k].w, bf));
+      }
+    }
+  };
+
+  // lane (co, h): taps 0..13 (h = 0) or 13..26 (h = 1); COB = 8 leaves half the lanes idle.  Rows of three taps each, and the
+  // middle row (dz, dy) = (1, 1), whose taps 0, 1 or 1, 2 the lane takes.
+  const int co = lane % COB, h = lane >> 4;
+  float acc[14];
+#pragma unroll
+  for (int j = 0; j < 14; ++j) acc[j] = 0.f;
+  auto consume = [&](const float* buf) {
+    const float* xc = buf + warp * XR * pitch;
+    const float* gc = buf + XR * CIC * pitch + co * gs;
+#pragma unroll 1
+    for (int r = 0; r < WG_ROWS; ++r) {
+      const float4* row[5];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int t = h ? k + 5 : k;   // row index 3 dz + dy
+        row[k] = reinterpret_cast<const float4*>(xc + ((t / 3) * (WG_ROWS + 2) + r + t % 3) * pitch);
+      }
+      row[4] = reinterpret_cast<const float4*>(xc + ((WG_ROWS + 2) + r + 1) * pitch);
+      const float4* g4 = reinterpret_cast<const float4*>(gc) + r * nq;
+      // window of voxels 4 q - 1 .. 4 q + 4 per row: pw, cur, nxt.x; the loads run one quad ahead
+      float pw[5];
+      float4 cur[5], nxt[5], g = g4[0];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        pw[k] = row[k][0].w;
+        cur[k] = row[k][1];
+        nxt[k] = row[k][2];
+      }
+#pragma unroll 3
+      for (int q = 0; q < nq; ++q) {   // the last quad's look-ahead reads past its row, unused
+        const float4 gn = g4[q + 1];
+        float4 ahead[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) ahead[k] = row[k][q + 3];
+        const float gv[4] = {g.x, g.y, g.z, g.w};
+        float w[5][6];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const float u[6] = {pw[k], cur[k].x, cur[k].y, cur[k].z, cur[k].w, nxt[k].x};
+#pragma unroll
+          for (int i = 0; i < 6; ++i) w[k][i] = u[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {   // voxel by voxel: 14 independent FMAs at a time
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) acc[3 * k + d] = fmaf(gv[i], w[k][i + d], acc[3 * k + d]);
+#pragma unroll
+          for (int d = 0; d < 2; ++d) acc[12 + d] = fmaf(gv[i], h ? w[4][i + d + 1] : w[4][i + d], acc[12 + d]);
+        }
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          pw[k] = cur[k].w;
+          cur[k] = nxt[k];
+          nxt[k] = ahead[k];
+        }
+        g = gn;
+      }
+    }
+  };
+
+  // two buffers: warps 4.. stage chunk i + 1 while warps 0..3 consume chunk i; one buffer: in turn
+  const bool consumer = warp < CIC, producer = warp >= 4;
+  const int nt = (int)blockDim.x;
+  const int pt = nbuf == 2 ? (int)threadIdx.x - 128 : (int)threadIdx.x, pn = nbuf == 2 ? nt - 128 : nt;
+  if (nbuf == 2) {
+    if (producer && (long long)blockIdx.x < chunks) stage(blockIdx.x, wg_sm, pt, pn);
+    __syncthreads();
+    int cur = 0;
+    for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+      if (producer) {
+        if (ch + gridDim.x < chunks) stage(ch + gridDim.x, wg_sm + (cur ^ 1) * buf_floats, pt, pn);
+      } else if (consumer) {
+        consume(wg_sm + cur * buf_floats);
+      }
+      __syncthreads();
+      cur ^= 1;
+    }
+  } else {
+    for (long long ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+      stage(ch, wg_sm, pt, pn);
+      __syncthreads();
+      if (consumer) consume(wg_sm);
+      __syncthreads();
+    }
+  }
+  if (consumer && ci0 + warp < ci_n && cob + co < co_n && (lane & 15) < COB) {
+    float* d = dW + ((long long)(cob + co) * ci_n + ci0 + warp) * 27;
+#pragma unroll
+    for (int j = 0; j < 12; ++j) atomicAdd(&d[h ? j + 15 : j], acc[j]);
+    if (!h) atomicAdd(&d[12], acc[12]);
+    atomicAdd(&d[h ? 14 : 13], acc[13]);   // tap 13 is in both halves: the first keeps it
+  }
+}
+
+// Shares of the volume per (input channel, 16 output channels): the length of a chain.
+static long long wgrad3_shares(int ci, int co, int B, int ny, int nz) {
+  const long long chunks = (long long)B * nz * ((ny + WG_ROWS - 1) / WG_ROWS);
+  const long long rest = (long long)ci * ((co + WG_CO - 1) / WG_CO);
+  return std::max(1LL, std::min(chunks, (4LL * 152 + rest - 1) / rest));
 }
 
 static cudaError_t wgrad3(const float* in, long long in_bs, int ci, const float* G, long long g_bs, int co, float* dW,
                           int B, int nx, int ny, int nz, int bf, cudaStream_t st) {
-  const size_t smem = sizeof(float) * (3 * (WG_ROWS + 2) * (nx + 2) + WG_CO * WG_ROWS * nx);
-  cudaError_t e = cudaFuncSetAttribute(k_wgrad3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr size_t kMax = 224 * 1024;   // beside the row table
+  const bool wide = wg_buf_floats(4, 16, nx) * 4 > kMax;   // rows above about 400 voxels: one channel by eight
+  const int cic = wide ? 1 : 4, cob = wide ? 8 : 16;
+  const size_t buf = wg_buf_floats(cic, cob, nx) * 4;
+  const int nbuf = 2 * buf <= kMax ? 2 : 1;
+  const size_t smem = nbuf * buf;
+  const bool vec = nx % 4 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)G % 16 == 0 && in_bs % 4 == 0 && g_bs % 4 == 0;
+  auto kern = wide ? (vec ? k_wgrad3<1, 8, true> : k_wgrad3<1, 8, false>) : (vec ? k_wgrad3<4, 16, true> : k_wgrad3<4, 16, false>);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const long long chunks = (long long)B * nz * ((ny + WG_ROWS - 1) / WG_ROWS);
-  const long long rest = (long long)ci * ((co + WG_CO - 1) / WG_CO);
-  const long long want = std::max(1LL, std::min(chunks, (4LL * 152 + rest - 1) / rest));
-  const dim3 grid((unsigned)want, ci, (co + WG_CO - 1) / WG_CO);
-  k_wgrad3<<<grid, WG_CO * 27, smem, st>>>(in, in_bs, ci, G, g_bs, co, dW, B, nx, ny, nz, bf);
+  const dim3 grid((unsigned)wgrad3_shares(ci, co, B, ny, nz), (ci + cic - 1) / cic, (co + cob - 1) / cob);
+  // one CTA per SM keeps twelve producer warps; more CTAs than SMs run two to an SM with four each
+  const int nt = (long long)grid.x * grid.y * grid.z > 152 ? 256 : WG_NT;
+  kern<<<grid, nt, smem, st>>>(in, in_bs, ci, G, g_bs, co, dW, B, nx, ny, nz, bf, nbuf);
   return cudaGetLastError();
 }
 
@@ -854,6 +1016,15 @@ extern "C" clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float*
 
 // conv3 backward for layer li: input `in` (ci channels, sample stride in_bs), output gradient
 // `g` (co channels, stride g_bs); writes din (if non-NULL) and accumulates dW.
+//
+// BF16 networks form dW on the tensor cores (16 -> 16 at 24 x 64x64x32: 0.29 ms, 1.46 ms on the
+// CUDA cores) unless the CUDA cores' FP32 chains are long: those round a sum of same-signed
+// terms further off than the tensor cores' short chains do, and a training run is meant to
+// keep following earlier ones.  The two differ by the square of the chain's length: at the
+// full-size level, whose activations carry the image's background, by up to 1.4e-5 of the
+// whole gradient at 41 k voxels a chain, at the coarser levels by 1.3e-6 at 79 k.  The
+// limits keep that at about 5e-6.
+constexpr long long kTcChainFull = 24LL << 10, kTcChainCoarse = 160LL << 10;
 static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long in_bs, const float* g, long long g_bs,
                               float* din, long long din_bs, int B, int nx, int ny, int nz, cudaStream_t st) {
   const Layer& L = u->layers[li];
@@ -863,7 +1034,11 @@ static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long 
     U_TRY(cudaGetLastError());
     U_TRY(conv3(bf, g, g_bs, L.co, din, din_bs, L.ci, u->flip, nullptr, false, B, nx, ny, nz, st, u->ctx()));
   }
-  U_TRY(wgrad3(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->bf, st));
+  const long long chain = li <= 1 || li >= 10 ? kTcChainFull : kTcChainCoarse;
+  if (u->ctx().on && (long long)B * nx * ny * nz <= chain * wgrad3_shares(L.ci, L.co, B, ny, nz))
+    U_TRY(clamp::unet_wgrad3_tc(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->err, st));
+  else
+    U_TRY(wgrad3(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->bf, st));
   return CLAMP_OK;
 }
 

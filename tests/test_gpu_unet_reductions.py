@@ -79,7 +79,8 @@ def _problem(ch, shape, B, seed):
 
 # FP32 network against exact gradients: 1e-4 as for the other FP32 gradient tests (FP32
 # forward and backward through twelve layers)
-@pytest.mark.parametrize("shape,B", [((4, 4, 4), 3), ((12, 4, 20), 2), ((4, 8, 136), 1), ((8, 36, 28), 5)])
+@pytest.mark.parametrize("shape,B", [((4, 4, 4), 3), ((12, 4, 20), 2), ((4, 8, 136), 1), ((8, 36, 28), 5),
+                                     ((4, 4, 256), 1), ((4, 8, 512), 1)])
 def test_fp32_gradients_match_oracle(C, shape, B):
     ch = (4, 8, 16)
     p, x, t = _problem(ch, shape, B, 41)
@@ -88,3 +89,22 @@ def test_fp32_gradients_match_oracle(C, shape, B):
     for i, (kind, ws, bs) in enumerate(_layers(ch)):
         assert rel(g[ws], gref[ws]) < 1e-4, (i, kind, "weights")
         assert rel(g[bs], gref[bs]) < 1e-4, (i, kind, "biases")
+
+
+# BF16 network whose 3x3x3 convs all run on the CUDA cores (no level is a width the tensor
+# convs take), so that both settings see the same activations and output gradients and only
+# the weight gradients' sums differ: FP32 chains and truncated 16-step tensor chains (3e-7 of
+# a same-signed sum) against each other.  1e-5 leaves 30x for cancellation within a layer.
+# Widths: below, at and above the 8, 16 and 32 voxel tiles, aligned and not; heights around
+# the rows of a tile.
+@pytest.mark.parametrize("shape,B,ch", [((4, 4, 4), 3, (4, 8, 16)), ((8, 12, 16), 2, (4, 8, 16)),
+                                        ((4, 20, 24), 3, (8, 16, 32)), ((12, 36, 20), 2, (16, 32, 64)),
+                                        ((8, 4, 40), 1, (16, 24, 40)), ((4, 68, 72), 2, (12, 20, 64))])
+def test_weight_gradients_tensor_cores_match_cuda_cores(C, shape, B, ch):
+    p, x, t = _problem(ch, shape, B, 61)
+    tc, cc = _grads(C, ch, p, x, t, "bf16", True), _grads(C, ch, p, x, t, "bf16", False)
+    for i, (kind, ws, bs) in enumerate(_layers(ch)):
+        assert np.isfinite(tc[ws]).all() and np.isfinite(tc[bs]).all()
+        assert rel(tc[ws], cc[ws]) < 1e-5, (i, kind, "weights", rel(tc[ws], cc[ws]))
+        assert rel(tc[bs], cc[bs]) < 1e-5, (i, kind, "biases", rel(tc[bs], cc[bs]))
+
