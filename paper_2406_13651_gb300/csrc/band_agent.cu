@@ -21,7 +21,7 @@
 // then gamma = S1 / (S2 / sigma_w^2 + S3) and the elementwise pass C.  Only P3 touches
 // every voxel: it reads mu, r' and writes d, plus two band rows.
 #include "clamp_kernels.cuh"
-#include "fft_core.cuh"
+#include "fft_reg.cuh"
 
 #include <math.h>
 
@@ -42,10 +42,11 @@ __device__ __forceinline__ float warp_sum_b(float v) {
   return v;
 }
 
-// FP32 per thread and warp, FP64 across warps in fixed order; writes out[k][idx].
-template <int NV>
+// FP32 per thread and warp, FP64 across the NTH / 32 warps in fixed order; writes out[k][idx].
+template <int NTH, int NV>
 __device__ __forceinline__ void block_sums(const float (&v)[NV], double* const (&out)[NV], long long idx) {
-  __shared__ double red[NT / 32][NV];
+  constexpr int NW = (NTH + 31) / 32;
+  __shared__ double red[NW][NV];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
@@ -55,7 +56,7 @@ __device__ __forceinline__ void block_sums(const float (&v)[NV], double* const (
   __syncthreads();
   if (threadIdx.x < NV) {
     double acc = 0.0;
-    for (int w = 0; w < NT / 32; ++w) acc += red[w][threadIdx.x];
+    for (int w = 0; w < NW; ++w) acc += red[w][threadIdx.x];
     out[threadIdx.x][idx] = acc;
   }
 }
@@ -123,111 +124,104 @@ __global__ void __launch_bounds__(1024) k_band_tables(const float* __restrict__ 
 // ---------------------------------------------------------------- P1: z pass on the support (inverse)
 
 template <int N>
-__global__ void __launch_bounds__(NT) k_band_z_inv(BandArgs a, const float2* __restrict__ tw) {
-  [[maybe_unused]] const long long nL = (long long)a.L * a.n, sL = (long long)a.L * a.nz * a.t.nSp,
-                                   bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
-  constexpr int LD = N + 1, CNT = BC * N, PER = (CNT + NT - 1) / NT;
+__global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_inv(BandArgs a, const float2* __restrict__ twB) {
+  [[maybe_unused]] const long long nL = (long long)a.L * a.n, sL = (long long)a.L * a.nz * a.t.nSp;   // buffer extents
+  constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2;
   float2* sm = reinterpret_cast<float2*>(band_smem);
-  const int s0 = blockIdx.x * BC, l = blockIdx.y;
-  const long long cbase = (long long)l * N * a.t.nSp + s0;   // compact [l][kz][s]
-  const long long ybase = (long long)l * a.n;
+  const int col = threadIdx.x % BC, j = threadIdx.x / BC;
+  const int s = blockIdx.x * BC + col, l = blockIdx.y;
+  const long long cbase = (long long)l * N * a.t.nSp + s;   // compact [l][kz][s]
   const float gp = a.gamma_prev ? __ldg(&a.gamma_prev[l]) : 0.0f;
-  float2 mv[PER], fv[PER], yv[PER];
-  float av[PER];
+  const bool valid = s < a.t.nS;   // padding columns hold stale values: read as zero
+  const bool step = valid && a.gamma_prev;
+  const float pup = __ldg(&a.t.s_pup[s]);
+  const long long ybase = (long long)l * a.n + __ldg(&a.t.s_kykx[s]);
+  float2 u[R2], fv[R2];
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int col = e % BC, kz = e / BC;
-      const long long ci = cbase + (long long)kz * a.t.nSp + col;
-      const int s = s0 + col;
-      const bool valid = s < a.t.nS;   // padding columns hold stale values: read as zero
-      mv[p] = valid && CLAMP_IN_BOUNDS(ci, sL, 101) ? a.Ms[ci] : make_float2(0.f, 0.f);
-      fv[p] = (valid && a.gamma_prev && CLAMP_IN_BOUNDS(ci, sL, 102)) ? a.Fd[ci] : make_float2(0.f, 0.f);
-      av[p] = __ldg(&a.t.s_pup[s]) * __ldg(&a.window[kz]);
-      const long long yi = ybase + (long long)kz * a.plane + __ldg(&a.t.s_kykx[s]);
-      yv[p] = CLAMP_IN_BOUNDS(yi, nL, 103) ? a.y[yi] : make_float2(0.f, 0.f);
-    }
+  for (int r = 0; r < R2; ++r) {
+    const long long ci = cbase + (long long)(j + r * R1) * a.t.nSp;
+    u[r] = valid && CLAMP_IN_BOUNDS(ci, sL, 101) ? a.Ms[ci] : make_float2(0.f, 0.f);
+    fv[r] = step && CLAMP_IN_BOUNDS(ci, sL, 102) ? a.Fd[ci] : make_float2(0.f, 0.f);
+  }
+  float2 yv[R2];
+#pragma unroll
+  for (int r = 0; r < R2; ++r) {
+    const long long yi = ybase + (long long)(j + r * R1) * a.plane;
+    yv[r] = CLAMP_IN_BOUNDS(yi, nL, 103) ? a.y[yi] : make_float2(0.f, 0.f);
   }
   float acc[1] = {0.f};
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int col = e % BC, kz = e / BC;
-      float2 M = mv[p];
-      if (a.gamma_prev && s0 + col < a.t.nS) {   // the previous step's spectrum update M += gamma F d
-        M.x = fmaf(gp, fv[p].x, M.x);
-        M.y = fmaf(gp, fv[p].y, M.y);
-        const long long mi = cbase + (long long)kz * a.t.nSp + col;
-        if (CLAMP_IN_BOUNDS(mi, sL, 104)) a.Ms[mi] = M;
-      }
-      const float f = av[p] * a.inv_nv;
-      sm[col * LD + kz] = make_float2(f * fmaf(-av[p], M.x, yv[p].x), f * fmaf(-av[p], M.y, yv[p].y));
-      acc[0] += av[p] * av[p] * cabs2(yv[p]);
+  for (int r = 0; r < R2; ++r) {
+    float2 M = u[r];
+    if (step) {   // the previous step's spectrum update M += gamma F d
+      M.x = fmaf(gp, fv[r].x, M.x);
+      M.y = fmaf(gp, fv[r].y, M.y);
+      const long long mi = cbase + (long long)(j + r * R1) * a.t.nSp;
+      if (CLAMP_IN_BOUNDS(mi, sL, 104)) a.Ms[mi] = M;
     }
+    const float av = pup * __ldg(&a.window[j + r * R1]), f = av * a.inv_nv;
+    u[r] = make_float2(f * fmaf(-av, M.x, yv[r].x), f * fmaf(-av, M.y, yv[r].y));
+    acc[0] += av * av * cabs2(yv[r]);
   }
-  __syncthreads();
-  fft_tile<N, BC, NT, true>(sm, tw);
+  rcol_first<N, true>(u, sm, col, j);
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int col = e % BC, z = e / BC;
-      const long long fi = cbase + (long long)z * a.t.nSp + col;
-      if (CLAMP_IN_BOUNDS(fi, sL, 105)) a.Fd[fi] = cscale(sm[col * LD + z], a.sc_z);   // Gz, in place
+  for (int i = 0; i < RCol<N>::NB; ++i) {
+    const int b = j + i * R1;
+    if (R2 % R1 != 0 && b >= R2) continue;
+    float2 v[R1];
+    rcol_second<N, true>(v, sm, col, b, twB);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const long long fi = cbase + (long long)(b + r * R2) * a.t.nSp;
+      if (CLAMP_IN_BOUNDS(fi, sL, 105)) a.Fd[fi] = cscale(v[r], a.sc_z);   // Gz, in place
     }
   }
   double* const outs[1] = {a.s4};
-  block_sums<1>(acc, outs, (long long)l * gridDim.x + blockIdx.x);
+  block_sums<RCol<N>::THREADS, 1>(acc, outs, (long long)l * gridDim.x + blockIdx.x);
 }
 
 // ---------------------------------------------------------------- P2 / P4: y passes on the band
 
 // INV: Gz on the support -> E on the band (zero off the support).  !INV: band -> support.
 template <int N, bool INV>
-__global__ void __launch_bounds__(NT) k_band_y(BandArgs a, const float2* __restrict__ tw) {
-  [[maybe_unused]] const long long nL = (long long)a.L * a.n, sL = (long long)a.L * a.nz * a.t.nSp,
+__global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_y(BandArgs a, const float2* __restrict__ twB) {
+  [[maybe_unused]] const long long sL = (long long)a.L * a.nz * a.t.nSp,
                                    bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
-  constexpr int LD = N + 1, CNT = BC * N, PER = (CNT + NT - 1) / NT;
+  constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2;
   float2* sm = reinterpret_cast<float2*>(band_smem);
-  const int b0 = blockIdx.x * BC, z = blockIdx.y, l = blockIdx.z;
-  const long long cplane = ((long long)l * a.nz + z) * a.t.nSp;             // compact [l][z][s]
-  const long long bbase = (((long long)l * a.nz + z) * N) * a.t.nbxp + b0;  // band [l][z][y][b]
-  float2 iv[PER];
+  const int col = threadIdx.x % BC, j = threadIdx.x / BC;
+  const int bc = blockIdx.x * BC + col, z = blockIdx.y, l = blockIdx.z;
+  const long long cplane = ((long long)l * a.nz + z) * a.t.nSp;               // compact [l][z][s]
+  const long long bbase = (((long long)l * a.nz + z) * N) * a.t.nbxp + bc;    // band [l][z][y][b]
+  float2 u[R2];
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int col = e % BC, yi = e / BC;
-      if constexpr (INV) {
-        const int s = __ldg(&a.t.sidx[yi * a.t.nbxp + b0 + col]);
-        iv[p] = s >= 0 && CLAMP_IN_BOUNDS(cplane + s, sL, 111) ? a.Fd[cplane + s] : make_float2(0.f, 0.f);
-      } else {
-        const long long bi = bbase + (long long)yi * a.t.nbxp + col;
-        iv[p] = CLAMP_IN_BOUNDS(bi, bL, 112) ? a.band[bi] : make_float2(0.f, 0.f);
-      }
+  for (int r = 0; r < R2; ++r) {
+    const int yi = j + r * R1;
+    if constexpr (INV) {
+      const int s = __ldg(&a.t.sidx[yi * a.t.nbxp + bc]);
+      u[r] = s >= 0 && CLAMP_IN_BOUNDS(cplane + s, sL, 111) ? a.Fd[cplane + s] : make_float2(0.f, 0.f);
+    } else {
+      const long long bi = bbase + (long long)yi * a.t.nbxp;
+      u[r] = CLAMP_IN_BOUNDS(bi, bL, 112) ? a.band[bi] : make_float2(0.f, 0.f);
     }
   }
+  rcol_first<N, INV>(u, sm, col, j);
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) sm[(e % BC) * LD + e / BC] = iv[p];
-  }
-  __syncthreads();
-  fft_tile<N, BC, NT, INV>(sm, tw);
+  for (int i = 0; i < RCol<N>::NB; ++i) {
+    const int b = j + i * R1;
+    if (R2 % R1 != 0 && b >= R2) continue;
+    float2 v[R1];
+    rcol_second<N, INV>(v, sm, col, b, twB);
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int col = e % BC, yi = e / BC;
-      const float2 v = cscale(sm[col * LD + yi], a.sc_y);
+    for (int r = 0; r < R1; ++r) {
+      const int yi = b + r * R2;
+      const float2 o = cscale(v[r], a.sc_y);
       if constexpr (INV) {
-        const long long bi = bbase + (long long)yi * a.t.nbxp + col;
-        if (CLAMP_IN_BOUNDS(bi, bL, 113)) a.band[bi] = v;
+        const long long bi = bbase + (long long)yi * a.t.nbxp;
+        if (CLAMP_IN_BOUNDS(bi, bL, 113)) a.band[bi] = o;
       } else {
-        const int s = __ldg(&a.t.sidx[yi * a.t.nbxp + b0 + col]);
-        if (s >= 0 && CLAMP_IN_BOUNDS(cplane + s, sL, 114)) a.Fd[cplane + s] = v;
+        const int s = __ldg(&a.t.sidx[yi * a.t.nbxp + bc]);
+        if (s >= 0 && CLAMP_IN_BOUNDS(cplane + s, sL, 114)) a.Fd[cplane + s] = o;
       }
     }
   }
@@ -239,99 +233,94 @@ enum BandRowMode { BAND_GRAD = 0, BAND_SPEC = 1 };
 
 // BAND_GRAD: e = inverse x-FFT of the band row, d = e - D mu (written), S1/S3, forward x-FFT
 // of d kept on the band.  BAND_SPEC: forward x-FFT of mu kept on the band (F mu's first axis).
-// Launch variant V = 0: rows_per_cta(N) rows per CTA, two CTAs per SM (at most 128
-// registers: with no occupancy bound the compiler takes about 180 and one CTA runs per SM,
-// 0.5 ms slower per iteration at 256x256x128, L = 32); V = 1: half as many rows, so a
-// thread holds half the prefetched values and three CTAs share an SM (at N = 256 with the
-// 8 x 8 x 4 radix plan, whose stages keep all threads of an 8-row tile busy); V = 2: the
-// tile of V = 0 with mu and r' not held in registers across the inverse transform: the CTA
-// first prefetches their lines into L2 (no registers held) and reads them after the
-// transform, so three CTAs share an SM.
+// A row's threads hold its voxels in registers between the two transforms (fft_reg.cuh), each
+// row within one warp: no block barrier, no tile staging.  Launch variant V = 0:
+// rows_per_cta(N) rows per CTA, two CTAs per SM; V = 1: half as many rows and threads, four
+// CTAs per SM (the same warps in smaller units); V = 2: mu and r' prefetched to L2 and read
+// after the inverse transform, so no registers hold them across it and three CTAs share an SM.
+template <int N, int V> struct RowCta {
+  static constexpr int THREADS = V == 1 ? NT / 2 : NT, LINES = THREADS / RRow<N>::T, MINB = V == 0 ? 2 : V == 1 ? 4 : 3;
+  static constexpr size_t SMEM = (size_t)LINES * RRow<N>::LS * sizeof(float2);
+  static_assert(LINES == (V == 1 ? variant_rows(N, 2) : rows_per_cta(N)), "rows per CTA");
+};
+
 template <int N, int MODE, int V>
-__global__ void __launch_bounds__(NT, V == 0 ? 2 : 3) k_band_x(BandArgs a, const float2* __restrict__ tw) {
-  [[maybe_unused]] const long long nL = (long long)a.L * a.n, sL = (long long)a.L * a.nz * a.t.nSp,
-                                   bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
-  constexpr int LX = V == 1 ? variant_rows(N, 2) : rows_per_cta(N), LD = N + 1, CNT = LX * N,
-                PER = (CNT + NT - 1) / NT;
+__global__ void __launch_bounds__(RowCta<N, V>::THREADS, RowCta<N, V>::MINB)
+    k_band_x(BandArgs a, const float2* __restrict__ twA, const float2* __restrict__ twB) {
+  [[maybe_unused]] const long long nL = (long long)a.L * a.n, bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
+  constexpr int R1 = RRow<N>::R1, R2 = RRow<N>::R2, T = RRow<N>::T, LINES = RowCta<N, V>::LINES;
   constexpr bool LATE = V == 2 && MODE == BAND_GRAD;   // mu, r' read after the inverse transform
-  using PL = std::conditional_t<V == 1 && N == 256, PlanB<N>, Plan<N>>;
-  float2* sm = reinterpret_cast<float2*>(band_smem);
-  const long long row0 = (long long)blockIdx.x * LX;   // rows over [L][nz][ny]
-  const long long e0 = row0 * N;
-  float2 mv[LATE ? 1 : PER], ev[PER];
-  float rv[LATE ? 1 : PER];
-  if constexpr (LATE) {   // 128-byte lines of the tile's mu (8 B per element) and r' (4 B)
-    static_assert(CNT % 32 == 0, "tile");
-    for (int i = threadIdx.x; i < CNT / 16; i += NT)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(a.mu + e0 + 16 * i));
-    for (int i = threadIdx.x; i < CNT / 32; i += NT)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(a.rprev + e0 + 32 * i));
+  const int line = threadIdx.x / T, j = threadIdx.x % T;
+  float2* sl = reinterpret_cast<float2*>(band_smem) + line * RRow<N>::LS;
+  const long long row0 = (long long)blockIdx.x * LINES;   // rows over [L][nz][ny]
+  const long long row = row0 + line, e0 = row * N + j, b0 = row * a.t.nbxp;
+  float2 mv[LATE ? 1 : R2];
+  float rv[LATE ? 1 : R2];
+  if constexpr (LATE) {   // the row's 128-byte lines of mu (8 B per element) and r' (4 B)
+    for (int i = j; i < N / 16; i += T) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.mu + row * N + 16 * i));
+    for (int i = j; i < N / 32; i += T) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.rprev + row * N + 32 * i));
   }
-  // with NT a multiple of N every element a thread touches is in the same column
-  constexpr bool FIXED_COL = NT % N == 0;
-  const int b_fixed = FIXED_COL && MODE == BAND_GRAD ? __ldg(&a.t.bpos[threadIdx.x % N]) : -1;
+  if constexpr (!LATE) {
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      if constexpr (!LATE) mv[p] = CLAMP_IN_BOUNDS(e0 + e, nL, 121) ? a.mu[e0 + e] : make_float2(0.f, 0.f);
-      if constexpr (MODE == BAND_GRAD) {
-        if constexpr (!LATE) rv[p] = CLAMP_IN_BOUNDS(e0 + e, nL, 122) ? a.rprev[e0 + e] : 1.0f;
-        const int line = e / N, i = e - line * N;
-        const int b = FIXED_COL ? b_fixed : __ldg(&a.t.bpos[i]);
-        ev[p] = b >= 0 && CLAMP_IN_BOUNDS((row0 + line) * a.t.nbxp + b, bL, 123) ? a.band[(row0 + line) * a.t.nbxp + b]
-                                                                               : make_float2(0.f, 0.f);
-      }
+    for (int r = 0; r < R2; ++r) {
+      mv[r] = CLAMP_IN_BOUNDS(e0 + r * R1, nL, 121) ? a.mu[e0 + r * R1] : make_float2(0.f, 0.f);
+      if constexpr (MODE == BAND_GRAD) rv[r] = CLAMP_IN_BOUNDS(e0 + r * R1, nL, 122) ? a.rprev[e0 + r * R1] : 1.0f;
     }
   }
-#pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int line = e / N, i = e - line * N;
-      sm[line * LD + i] = MODE == BAND_GRAD ? ev[p] : mv[LATE ? 0 : p];
-    }
-  }
-  __syncthreads();
   float acc[2] = {0.f, 0.f};
+  float2 u[R2];
   if constexpr (MODE == BAND_GRAD) {
-    fft_tile<N, LX, NT, true, PL>(sm, tw);
 #pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const int e = threadIdx.x + p * NT;
-      if (CNT % NT == 0 || e < CNT) {
-        const int line = e / N, i = e - line * N;
-        const float2 ee = cscale(sm[line * LD + i], a.sc_x);
-        const bool ok = !LATE || CLAMP_IN_BOUNDS(e0 + e, nL, 124);
-        const float2 m = LATE ? (ok ? a.mu[e0 + e] : make_float2(0.f, 0.f)) : mv[LATE ? 0 : p];
-        const float D = __frcp_rn((LATE ? (ok ? a.rprev[e0 + e] : 1.0f) : rv[LATE ? 0 : p]) + a.floor);
-        const float2 dv = make_float2(fmaf(-D, m.x, ee.x), fmaf(-D, m.y, ee.y));
-        if (CLAMP_IN_BOUNDS(e0 + e, nL, 126)) a.d[e0 + e] = dv;
-        const float d2 = cabs2(dv);
-        acc[0] += d2;
-        acc[1] += D * d2;
-        sm[line * LD + i] = dv;
+    for (int i = 0; i < RRow<N>::NB; ++i) {
+      const int b = j + i * T;
+      if (R2 % T != 0 && b >= R2) continue;
+      float2 v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) {
+        const int bp = __ldg(&a.t.bpos[b + r * R2]);
+        v[r] = bp >= 0 && CLAMP_IN_BOUNDS(b0 + bp, bL, 123) ? a.band[b0 + bp] : make_float2(0.f, 0.f);
       }
+      rrow_inv_outer<N>(v, sl, b);
     }
-    __syncthreads();
+    __syncwarp();
+    rrow_inv_mid<N>(u, sl, j, twA);
+#pragma unroll
+    for (int r = 0; r < R2; ++r) {
+      const long long e = e0 + r * R1;
+      const bool ok = !LATE || CLAMP_IN_BOUNDS(e, nL, 124);
+      const float2 m = LATE ? (ok ? a.mu[e] : make_float2(0.f, 0.f)) : mv[LATE ? 0 : r];
+      const float D = __frcp_rn((LATE ? (ok ? a.rprev[e] : 1.0f) : rv[LATE ? 0 : r]) + a.floor);
+      const float2 dv = make_float2(fmaf(-D, m.x, u[r].x * a.sc_x), fmaf(-D, m.y, u[r].y * a.sc_x));
+      if (CLAMP_IN_BOUNDS(e, nL, 126)) a.d[e] = dv;
+      const float d2 = cabs2(dv);
+      acc[0] += d2;
+      acc[1] += D * d2;
+      u[r] = dv;
+    }
+    __syncwarp();   // the line's reads of the exchange are done
+  } else {
+#pragma unroll
+    for (int r = 0; r < R2; ++r) u[r] = mv[LATE ? 0 : r];
   }
-  fft_tile<N, LX, NT, false, PL>(sm, tw);
-  // band of the forward transform: LX rows x nbxp columns (padding columns get zeros)
-  // (a warp per row at a time, lanes over the band columns: no division by nbxp)
-  const int nbxp = a.t.nbxp;
-  for (int line = threadIdx.x >> 5; line < LX; line += NT / 32) {
-    float2* brow = a.band + (row0 + line) * nbxp;
-    for (int b = threadIdx.x & 31; b < nbxp; b += 32) {
-      const int kx = __ldg(&a.t.bx[b]);
-      if (CLAMP_IN_BOUNDS((row0 + line) * nbxp + b, bL, 127))
-        brow[b] = kx >= 0 ? cscale(sm[line * LD + kx], a.sc_x) : make_float2(0.f, 0.f);
+  rrow_fwd_mid<N>(u, sl, j);
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < RRow<N>::NB; ++i) {
+    const int b = j + i * T;
+    if (R2 % T != 0 && b >= R2) continue;
+    float2 v[R1];
+    rrow_fwd_outer<N>(v, sl, b, twB);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {   // the band's padding columns stay as they are: nothing reads them
+      const int bp = __ldg(&a.t.bpos[b + r * R2]);
+      if (bp >= 0 && CLAMP_IN_BOUNDS(b0 + bp, bL, 127)) a.band[b0 + bp] = cscale(v[r], a.sc_x);
     }
   }
   if constexpr (MODE == BAND_GRAD) {
     double* const outs[2] = {a.s1, a.s3};
     const long long rows_per_look = (long long)a.nz * a.ny;
     const long long look = row0 / rows_per_look;
-    block_sums<2>(acc, outs, look * a.px + (row0 - look * rows_per_look) / LX);
+    block_sums<RowCta<N, V>::THREADS, 2>(acc, outs, look * a.px + (row0 - look * rows_per_look) / LINES);
   }
 }
 
@@ -339,49 +328,45 @@ __global__ void __launch_bounds__(NT, V == 0 ? 2 : 3) k_band_x(BandArgs a, const
 
 // BAND_GRAD: F d on the support (in place) and S2 = ||a F d||^2.  BAND_SPEC: writes M.
 template <int N, int MODE>
-__global__ void __launch_bounds__(NT) k_band_z_fwd(BandArgs a, const float2* __restrict__ tw) {
-  [[maybe_unused]] const long long nL = (long long)a.L * a.n, sL = (long long)a.L * a.nz * a.t.nSp,
-                                   bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
-  constexpr int LD = N + 1, CNT = BC * N, PER = (CNT + NT - 1) / NT;
+__global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_fwd(BandArgs a, const float2* __restrict__ twB) {
+  [[maybe_unused]] const long long sL = (long long)a.L * a.nz * a.t.nSp;   // buffer extent
+  constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2;
   float2* sm = reinterpret_cast<float2*>(band_smem);
-  const int s0 = blockIdx.x * BC, l = blockIdx.y;
-  const long long cbase = (long long)l * N * a.t.nSp + s0;
-  float2 iv[PER];
+  const int col = threadIdx.x % BC, j = threadIdx.x / BC;
+  const int s = blockIdx.x * BC + col, l = blockIdx.y;
+  const long long cbase = (long long)l * N * a.t.nSp + s;
+  const bool valid = s < a.t.nS;
+  float2 u[R2];
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const long long fi = cbase + (long long)(e / BC) * a.t.nSp + e % BC;
-      iv[p] = s0 + e % BC < a.t.nS && CLAMP_IN_BOUNDS(fi, sL, 131) ? a.Fd[fi] : make_float2(0.f, 0.f);
-    }
+  for (int r = 0; r < R2; ++r) {
+    const long long fi = cbase + (long long)(j + r * R1) * a.t.nSp;
+    u[r] = valid && CLAMP_IN_BOUNDS(fi, sL, 131) ? a.Fd[fi] : make_float2(0.f, 0.f);
   }
-#pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) sm[(e % BC) * LD + e / BC] = iv[p];
-  }
-  __syncthreads();
-  fft_tile<N, BC, NT, false>(sm, tw);
+  rcol_first<N, false>(u, sm, col, j);
   float acc[1] = {0.f};
 #pragma unroll
-  for (int p = 0; p < PER; ++p) {
-    const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int col = e % BC, kz = e / BC;
-      const float2 v = cscale(sm[col * LD + kz], a.sc_z);
-      const long long ci = cbase + (long long)kz * a.t.nSp + col;
+  for (int i = 0; i < RCol<N>::NB; ++i) {
+    const int b = j + i * R1;
+    if (R2 % R1 != 0 && b >= R2) continue;
+    float2 v[R1];
+    rcol_second<N, false>(v, sm, col, b, twB);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const int kz = b + r * R2;
+      const float2 o = cscale(v[r], a.sc_z);
+      const long long ci = cbase + (long long)kz * a.t.nSp;
       if constexpr (MODE == BAND_GRAD) {
-        if (CLAMP_IN_BOUNDS(ci, sL, 132)) a.Fd[ci] = v;
-        const float av = __ldg(&a.t.s_pup[s0 + col]) * __ldg(&a.window[kz]);
-        acc[0] += av * av * cabs2(v);
+        if (CLAMP_IN_BOUNDS(ci, sL, 132)) a.Fd[ci] = o;
+        const float av = __ldg(&a.t.s_pup[s]) * __ldg(&a.window[kz]);
+        acc[0] += av * av * cabs2(o);
       } else {
-        if (CLAMP_IN_BOUNDS(ci, sL, 133)) a.Ms[ci] = v;
+        if (CLAMP_IN_BOUNDS(ci, sL, 133)) a.Ms[ci] = o;
       }
     }
   }
   if constexpr (MODE == BAND_GRAD) {
     double* const outs[1] = {a.s2};
-    block_sums<1>(acc, outs, (long long)l * gridDim.x + blockIdx.x);
+    block_sums<RCol<N>::THREADS, 1>(acc, outs, (long long)l * gridDim.x + blockIdx.x);
   }
 }
 
@@ -437,74 +422,49 @@ cudaError_t dispatch_n(int N, F&& f) {
     if (_e != cudaSuccess) return _e; \
   } while (0)
 
-template <class K>
-cudaError_t smem_attr(K kern, size_t smem) {
-  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 cudaError_t run_z(const BandArgs& a, int L, bool inverse, int mode, cudaStream_t st) {
   return dispatch_n(a.nz, [&](auto NC) -> cudaError_t {
-    constexpr int N = decltype(NC)::value;
-    const size_t smem = (size_t)BC * (N + 1) * sizeof(float2);
+    constexpr int N = decltype(NC)::value, TH = RCol<N>::THREADS;
+    constexpr size_t smem = RCol<N>::SMEM;   // at most 33 KB: within the default limit
     const dim3 grid(a.t.nSp / BC, L);
-    if (inverse) {
-      BAND_TRY(smem_attr(k_band_z_inv<N>, smem));
-      k_band_z_inv<N><<<grid, NT, smem, st>>>(a, twiddle_table(N));
-    } else if (mode == BAND_GRAD) {
-      BAND_TRY(smem_attr(k_band_z_fwd<N, BAND_GRAD>, smem));
-      k_band_z_fwd<N, BAND_GRAD><<<grid, NT, smem, st>>>(a, twiddle_table(N));
-    } else {
-      BAND_TRY(smem_attr(k_band_z_fwd<N, BAND_SPEC>, smem));
-      k_band_z_fwd<N, BAND_SPEC><<<grid, NT, smem, st>>>(a, twiddle_table(N));
-    }
+    if (inverse) k_band_z_inv<N><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
+    else if (mode == BAND_GRAD) k_band_z_fwd<N, BAND_GRAD><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
+    else k_band_z_fwd<N, BAND_SPEC><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
     return cudaGetLastError();
   });
 }
 
 cudaError_t run_y(const BandArgs& a, int L, bool inverse, cudaStream_t st) {
   return dispatch_n(a.ny, [&](auto NC) -> cudaError_t {
-    constexpr int N = decltype(NC)::value;
-    const size_t smem = (size_t)BC * (N + 1) * sizeof(float2);
+    constexpr int N = decltype(NC)::value, TH = RCol<N>::THREADS;
+    constexpr size_t smem = RCol<N>::SMEM;
     const dim3 grid(a.t.nbxp / BC, a.nz, L);
-    if (inverse) {
-      BAND_TRY(smem_attr(k_band_y<N, true>, smem));
-      k_band_y<N, true><<<grid, NT, smem, st>>>(a, twiddle_table(N));
-    } else {
-      BAND_TRY(smem_attr(k_band_y<N, false>, smem));
-      k_band_y<N, false><<<grid, NT, smem, st>>>(a, twiddle_table(N));
-    }
+    if (inverse) k_band_y<N, true><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
+    else k_band_y<N, false><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
     return cudaGetLastError();
   });
+}
+
+template <int N, int MODE, int V>
+cudaError_t launch_x(const BandArgs& a, int L, cudaStream_t st) {
+  using Cta = RowCta<N, V>;
+  static_assert(Cta::SMEM <= 48 * 1024, "default shared-memory limit");
+  const unsigned grid = (unsigned)((long long)L * a.nz * a.ny / Cta::LINES);
+  k_band_x<N, MODE, V><<<grid, Cta::THREADS, Cta::SMEM, st>>>(a, twiddle_table_a(N), twiddle_table_b(N));
+  return cudaGetLastError();
 }
 
 cudaError_t run_x(const BandArgs& a, int L, int mode, int variant, cudaStream_t st) {
   return dispatch_n(a.nx, [&](auto NC) -> cudaError_t {
     constexpr int N = decltype(NC)::value;
-    if (mode == BAND_GRAD && variant == 1) {
-      constexpr int LX = variant_rows(N, 2);
-      const size_t smem = (size_t)LX * (N + 1) * sizeof(float2);
-      BAND_TRY(smem_attr(k_band_x<N, BAND_GRAD, 1>, smem));
-      k_band_x<N, BAND_GRAD, 1><<<(unsigned)((long long)L * a.nz * a.ny / LX), NT, smem, st>>>(a, twiddle_table(N));
-      return cudaGetLastError();
-    }
-    if (mode == BAND_GRAD && variant == 2) {
-      constexpr int LX = rows_per_cta(N);
-      const size_t smem = (size_t)LX * (N + 1) * sizeof(float2);
-      BAND_TRY(smem_attr(k_band_x<N, BAND_GRAD, 2>, smem));
-      k_band_x<N, BAND_GRAD, 2><<<(unsigned)((long long)L * a.nz * a.ny / LX), NT, smem, st>>>(a, twiddle_table(N));
-      return cudaGetLastError();
-    }
-    constexpr int LX = rows_per_cta(N);
-    const size_t smem = (size_t)LX * (N + 1) * sizeof(float2);
-    const unsigned grid = (unsigned)((long long)L * a.nz * a.ny / LX);
-    if (mode == BAND_GRAD) {
-      BAND_TRY(smem_attr(k_band_x<N, BAND_GRAD, 0>, smem));
-      k_band_x<N, BAND_GRAD, 0><<<grid, NT, smem, st>>>(a, twiddle_table(N));
+    if constexpr (N < 16) {   // nx is a multiple of 16
+      return cudaErrorInvalidValue;
     } else {
-      BAND_TRY(smem_attr(k_band_x<N, BAND_SPEC, 0>, smem));
-      k_band_x<N, BAND_SPEC, 0><<<grid, NT, smem, st>>>(a, twiddle_table(N));
+      if (mode == BAND_SPEC) return launch_x<N, BAND_SPEC, 0>(a, L, st);
+      if (variant == 1) return launch_x<N, BAND_GRAD, 1>(a, L, st);
+      if (variant == 2) return launch_x<N, BAND_GRAD, 2>(a, L, st);
+      return launch_x<N, BAND_GRAD, 0>(a, L, st);
     }
-    return cudaGetLastError();
   });
 }
 

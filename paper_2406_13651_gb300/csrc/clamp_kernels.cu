@@ -15,6 +15,7 @@
 // the App. A prox and the Mann step.
 #include "clamp_kernels.cuh"
 #include "fft_core.cuh"
+#include "fft_reg.cuh"
 
 #include <math.h>
 
@@ -24,6 +25,7 @@
 namespace clamp {
 
 __device__ float2 g_tw[kTwTotal];
+__device__ float2 g_tw2[2 * kTwTotal];   // fft_reg.cuh's tables: A, then B
 
 cudaError_t upload_twiddles() {
   std::vector<float2> h(kTwTotal);
@@ -34,6 +36,15 @@ cudaError_t upload_twiddles() {
       h[off + m] = make_float2((float)cos(ang), (float)sin(ang));
     }
   }
+  std::vector<float2> h2(2 * kTwTotal);
+  for (int N : kFftLengths)
+    for (int t = 0; t < 2; ++t) {
+      const int ns = t == 0 ? rplan_r1(N) : N / rplan_r1(N);   // first radix of the plan
+      for (int r = 0; r < N / ns; ++r)
+        for (int k = 0; k < ns; ++k) h2[t * kTwTotal + tw_offset(N) + r * ns + k] = h[tw_offset(N) + r * k];
+    }
+  const cudaError_t e = cudaMemcpyToSymbol(g_tw2, h2.data(), sizeof(float2) * h2.size());
+  if (e != cudaSuccess) return e;
   return cudaMemcpyToSymbol(g_tw, h.data(), sizeof(float2) * kTwTotal);
 }
 
@@ -44,6 +55,13 @@ static const float2* tw_ptr(int N) {
 }
 
 const float2* twiddle_table(int N) { return tw_ptr(N); }
+
+const float2* twiddle_table_a(int N) {
+  void* p = nullptr;
+  cudaGetSymbolAddress(&p, g_tw2);
+  return reinterpret_cast<const float2*>(p) + tw_offset(N);
+}
+const float2* twiddle_table_b(int N) { return twiddle_table_a(N) + kTwTotal; }
 
 extern __shared__ float4 dyn_smem[];
 

@@ -93,6 +93,9 @@ struct Partials {
 cudaError_t upload_twiddles();
 // Device address of the length-N twiddle table (N a supported axis length).
 const float2* twiddle_table(int N);
+// The register FFTs' tables (fft_reg.cuh).
+const float2* twiddle_table_a(int N);
+const float2* twiddle_table_b(int N);
 
 // ---- band-limited forward agent (band_agent.cu): the gradient's transforms on the
 // aperture's support only.  Support S = {(ky, kx): pupil != 0} (row by row), band
