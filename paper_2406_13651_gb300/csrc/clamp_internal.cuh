@@ -48,6 +48,11 @@ size_t unet_conv3_tc_wpk_bytes(int ci, int co);
 cudaError_t unet_conv3_tc(const float* in, long long in_bs, int ci, float* out, long long out_bs, int co,
                           const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz, uint4* wpk,
                           int* err, cudaStream_t st);
+// The same conv on the CUDA cores, any channel counts and sizes: FP32 chains in the order (input
+// channel, tap); bf rounds both operands to BF16.
+cudaError_t unet_conv3_cc(bool bf, const float* in, long long in_bs, int ci, float* out, long long out_bs, int co,
+                          const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz,
+                          cudaStream_t st);
 // dW[co][ci][27] += sum over samples and voxels of G[co][v] in[ci][v + tap] with both operands
 // rounded to BF16, on the tensor cores (any channel counts and volume).  err as above.
 cudaError_t unet_wgrad3_tc(const float* in, long long in_bs, int ci, const float* G, long long g_bs, int co, float* dW,

@@ -23,11 +23,6 @@ namespace unet {
 constexpr int UT = 256;
 
 // BF16 mode: an operand rounded to bfloat16 (round to nearest even) and widened back.
-template <bool BF>
-__device__ __forceinline__ float opnd(float x) {
-  if constexpr (BF) return __bfloat162float(__float2bfloat16_rn(x));
-  else return x;
-}
 __device__ __forceinline__ float opr(float x, int bf) {
   return bf ? __bfloat162float(__float2bfloat16_rn(x)) : x;
 }
@@ -39,115 +34,6 @@ struct Layer {
   size_t nw;    // weight count
 };
 
-// ---------------------------------------------------------------- 3x3x3 conv (forward and dgrad)
-
-constexpr int CX = 32, CVX = 4;  // output x per CTA, per thread
-
-// out[b][co][v] = bias[co] + sum_ci sum_tap W[co][ci][tap] in[b][ci][v + tap] (zero padding), optional ReLU.
-// in / out address sample b at in + b * in_bs, channel c at + c * n.
-template <int CO, int CG, int CINC, bool BF>
-__global__ void __launch_bounds__(UT) k_conv3(const float* __restrict__ in, long long in_bs, int ci_n,
-                                              float* __restrict__ out, long long out_bs, int co_n,
-                                              const float* __restrict__ W, const float* __restrict__ bias, int relu,
-                                              int nx, int ny, int nz) {
-  constexpr int TY = UT / ((CX / CVX) * CG), IX = CX + 2, IY = TY + 2, COT = CO * CG;
-  __shared__ float s_in[CINC * 3 * IY * IX];
-  __shared__ float s_w[CINC * 27 * COT];
-  const int tx = threadIdx.x % (CX / CVX);
-  const int ty = (threadIdx.x / (CX / CVX)) % TY;
-  const int cg = threadIdx.x / ((CX / CVX) * TY);
-  const int x0 = blockIdx.x * CX, y0 = blockIdx.y * TY;
-  const int ncb = (co_n + COT - 1) / COT;
-  const int zz = blockIdx.z / ncb, cb = blockIdx.z % ncb;
-  const int b = zz / nz, z = zz % nz;
-  const long long plane = (long long)nx * ny, n = plane * nz;
-  const float* inb = in + (long long)b * in_bs;
-  float acc[CVX][CO];
-#pragma unroll
-  for (int o = 0; o < CO; ++o) {
-    const int co = cb * COT + cg * CO + o;
-    const float bv = (bias && co < co_n) ? __ldg(&bias[co]) : 0.f;
-#pragma unroll
-    for (int v = 0; v < CVX; ++v) acc[v][o] = bv;
-  }
-  for (int c0 = 0; c0 < ci_n; c0 += CINC) {
-    __syncthreads();
-    for (int e = threadIdx.x; e < CINC * 3 * IY * IX; e += UT) {
-      const int xi = e % IX, yi = (e / IX) % IY, zi = (e / (IX * IY)) % 3, ci = e / (IX * IY * 3);
-      const int gx = x0 + xi - 1, gy = y0 + yi - 1, gz = z + zi - 1;
-      float v = 0.f;
-      if (c0 + ci < ci_n && gx >= 0 && gx < nx && gy >= 0 && gy < ny && gz >= 0 && gz < nz)
-        v = __ldg(&inb[(long long)(c0 + ci) * n + (long long)gz * plane + (long long)gy * nx + gx]);
-      s_in[e] = opnd<BF>(v);
-    }
-    for (int e = threadIdx.x; e < CINC * 27 * COT; e += UT) {
-      const int o = e % COT, tap = (e / COT) % 27, ci = e / (COT * 27);
-      const int co = cb * COT + o;
-      s_w[e] = (co < co_n && c0 + ci < ci_n) ? opnd<BF>(__ldg(&W[((long long)co * ci_n + c0 + ci) * 27 + tap])) : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int ci = 0; ci < CINC; ++ci) {
-#pragma unroll
-      for (int dz = 0; dz < 3; ++dz) {
-#pragma unroll
-        for (int dy = 0; dy < 3; ++dy) {
-          const float* row = s_in + ((ci * 3 + dz) * IY + ty + dy) * IX + tx * CVX;
-          float xin[CVX + 2];
-#pragma unroll
-          for (int q = 0; q < CVX + 2; ++q) xin[q] = row[q];
-#pragma unroll
-          for (int dx = 0; dx < 3; ++dx) {
-            const float* wp = s_w + (ci * 27 + dz * 9 + dy * 3 + dx) * COT + cg * CO;
-#pragma unroll
-            for (int o = 0; o < CO; ++o) {
-              const float wv = wp[o];
-#pragma unroll
-              for (int v = 0; v < CVX; ++v) acc[v][o] = fmaf(xin[v + dx], wv, acc[v][o]);
-            }
-          }
-        }
-      }
-    }
-  }
-  const int gy = y0 + ty;
-  if (gy >= ny) return;
-  float* outb = out + (long long)b * out_bs;
-#pragma unroll
-  for (int o = 0; o < CO; ++o) {
-    const int co = cb * COT + cg * CO + o;
-    if (co >= co_n) continue;
-#pragma unroll
-    for (int v = 0; v < CVX; ++v) {
-      const int gx = x0 + tx * CVX + v;
-      if (gx >= nx) continue;
-      float r = acc[v][o];
-      if (relu) r = fmaxf(r, 0.f);
-      outb[(long long)co * n + (long long)z * plane + (long long)gy * nx + gx] = r;
-    }
-  }
-}
-
-template <bool BF>
-static void conv3_launch(const float* in, long long in_bs, int ci, float* out, long long out_bs, int co,
-                         const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz, cudaStream_t st) {
-  constexpr int CO = 8;
-  if (co <= 16) {
-    constexpr int CG = 2, TY = UT / ((CX / CVX) * CG);
-    dim3 grid((nx + CX - 1) / CX, (ny + TY - 1) / TY, B * nz * ((co + CO * CG - 1) / (CO * CG)));
-    if (ci == 1)
-      k_conv3<CO, CG, 1, BF><<<grid, UT, 0, st>>>(in, in_bs, ci, out, out_bs, co, W, bias, relu, nx, ny, nz);
-    else
-      k_conv3<CO, CG, 4, BF><<<grid, UT, 0, st>>>(in, in_bs, ci, out, out_bs, co, W, bias, relu, nx, ny, nz);
-  } else {
-    constexpr int CG = 4, TY = UT / ((CX / CVX) * CG);
-    dim3 grid((nx + CX - 1) / CX, (ny + TY - 1) / TY, B * nz * ((co + CO * CG - 1) / (CO * CG)));
-    if (ci == 1)
-      k_conv3<CO, CG, 1, BF><<<grid, UT, 0, st>>>(in, in_bs, ci, out, out_bs, co, W, bias, relu, nx, ny, nz);
-    else
-      k_conv3<CO, CG, 4, BF><<<grid, UT, 0, st>>>(in, in_bs, ci, out, out_bs, co, W, bias, relu, nx, ny, nz);
-  }
-}
 // Tensor-core path of a network (BF16 only): packed-weight scratch, error word, switch.
 struct TcCtx {
   uint4* wpk;
@@ -160,16 +46,7 @@ static cudaError_t conv3(bool bf, const float* in, long long in_bs, int ci, floa
                          const TcCtx& tc) {
   if (bf && tc.on && unet_conv3_tc_supported(ci, co, nx, ny))
     return unet_conv3_tc(in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, tc.wpk, tc.err, st);
-  // grid.z = samples * nz * channel blocks must stay <= 65535: launch sample chunks
-  const int per = std::max(1, 65535 / (nz * ((co + 15) / 16)));
-  for (int b0 = 0; b0 < B; b0 += per) {
-    const int bc = std::min(per, B - b0);
-    const float* i0 = in + (long long)b0 * in_bs;
-    float* o0 = out + (long long)b0 * out_bs;
-    if (bf) conv3_launch<true>(i0, in_bs, ci, o0, out_bs, co, W, bias, relu, bc, nx, ny, nz, st);
-    else conv3_launch<false>(i0, in_bs, ci, o0, out_bs, co, W, bias, relu, bc, nx, ny, nz, st);
-  }
-  return cudaGetLastError();
+  return unet_conv3_cc(bf, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st);
 }
 
 // W'[ci][co][26 - tap] = W[co][ci][tap]: the dgrad of a 3x3x3 conv is the conv of the output

@@ -1,0 +1,234 @@
+// unet_conv.cu -- the U-Net's 3x3x3 convolutions on the CUDA cores: FP32 networks, the first
+// layer (one input channel) and the levels whose rows are no whole tensor-core tiles; the
+// forward conv and, with flipped weights, the data gradient.
+//
+//     out[b][co][v] = bias[co] + sum_ci sum_tap W[co][ci][tap] in[b][ci][v + tap]
+// (zero padding, optional ReLU), one FP32 chain per output in the order ci, dz, dy, dx.
+//
+// A thread holds 4 x voxels x 8 output channels; the accumulators of two channels are one
+// packed pair, so an FFMA2 (fma.rn.f32x2: each half rounded as fmaf rounds) does two terms
+// and a (row, 3 taps) step is 48 of them beside six 16-byte weight loads, two input loads
+// and the packing of six inputs.  A CTA owns TY rows of CX voxels of one plane and 8 CG
+// channels; the widths 8, 16 and 32 are chosen by what the level's rows leave unused.  Per
+// input channel its three planes and its weights are staged once, the next channel's loads
+// in flight in registers while the current one's FMAs run (two buffers, one barrier per
+// channel).  Weights come straight from W: runs of 27 taps, transposed on the way to shared
+// memory, so a network in use on several streams needs no shared scratch.
+//
+// Bound by the FMA pipe and the issue of its loads (64 -> 64 at 48x48x24: 165 us of FMAs).  The
+// kernel before it had one tile width (32: a quarter of a 48-wide level's and three quarters of
+// an 8-wide level's threads idle), scalar FMAs and nothing in flight while it staged: warm
+// start at 192x192x96 2.92 -> 2.42 ms (its two 48x48x24 convs 0.87 -> about 0.37), training step
+// on 24 x 32^3 5.02 -> 4.13 ms (its four at 8^3), the first layer at 256x256x128 0.33 -> 0.23 ms.
+#include "../../include/clamp.h"
+#include "clamp_internal.cuh"
+#include "clamp_kernels.cuh"
+
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+namespace clamp {
+namespace unet_cc {
+
+typedef unsigned long long f2;   // two packed FP32
+
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// BF16 mode: an operand rounded to bfloat16 (round to nearest even) and widened back.
+template <bool BF>
+__device__ __forceinline__ float opnd(float x) {
+  if constexpr (BF) return __bfloat162float(__float2bfloat16_rn(x));
+  else return x;
+}
+
+// CX: x voxels of a tile, CG: groups of 8 output channels.
+template <int CX, int CG>
+struct CcCfg {
+  static constexpr int TX = CX / 4, TY = CG == 2 ? 16 : CX == 32 && CG == 8 ? 4 : 8;
+  static constexpr int THREADS = TX * TY * CG;
+  static constexpr int COT = 8 * CG, WP = COT + 8;                 // channels, weight row pitch (conflict-free stores)
+  static constexpr int IX = CX + 2, IY = TY + 2, IP = CX + 4;      // staged rows, row pitch (16-byte aligned rows)
+  static constexpr int NIN = (3 * IY * IX + THREADS - 1) / THREADS;
+  static constexpr int TPC = THREADS / COT, NW = (27 + TPC - 1) / TPC;   // threads per channel's weights, taps each
+  static constexpr int MINB = 512 / THREADS;                       // 16 warps per SM: up to 128 registers
+};
+
+template <int CX, int CG, bool BF>
+__global__ void __launch_bounds__(CcCfg<CX, CG>::THREADS, CcCfg<CX, CG>::MINB)
+    k_conv3(const float* __restrict__ in, long long in_bs, int ci_n, float* __restrict__ out, long long out_bs,
+            int co_n, const float* __restrict__ W, const float* __restrict__ bias, int relu, int nx, int ny, int nz,
+            int vec) {
+  using Cfg = CcCfg<CX, CG>;
+  constexpr int T = Cfg::THREADS, TX = Cfg::TX, TY = Cfg::TY, IX = Cfg::IX, IY = Cfg::IY, IP = Cfg::IP, WP = Cfg::WP;
+  __shared__ __align__(16) float s_in[2][3 * IY * IP];
+  __shared__ __align__(16) float s_w[2][27 * WP];
+  const int tid = threadIdx.x;
+  const int tx = tid % TX, ty = (tid / TX) % TY, cg = tid / (TX * TY);
+  const int x0 = blockIdx.x * CX, y0 = blockIdx.y * TY;
+  const int ncb = (co_n + Cfg::COT - 1) / Cfg::COT;
+  const int zz = blockIdx.z / ncb, co0 = (int)(blockIdx.z % ncb) * Cfg::COT;
+  const int b = zz / nz, z = zz % nz;
+  const long long plane = (long long)nx * ny, n = plane * nz;
+
+  // what this thread stages of a channel: voxels (offset from the tile's first, in[] valid) and weights
+  const float* inb = in + (long long)b * in_bs + z * plane + (long long)y0 * nx + x0;
+  long long off[Cfg::NIN];
+  unsigned valid = 0;
+#pragma unroll
+  for (int k = 0; k < Cfg::NIN; ++k) {
+    const int e = tid + k * T, xi = e % IX - 1, yi = e / IX % IY - 1, zi = e / (IX * IY) - 1;
+    const int gx = x0 + xi, gy = y0 + yi, gz = z + zi;
+    const bool ok = e < 3 * IY * IX && gx >= 0 && gx < nx && gy >= 0 && gy < ny && gz >= 0 && gz < nz;
+    off[k] = ok ? zi * plane + (long long)yi * nx + xi : 0;
+    valid |= (ok ? 1u : 0u) << k;
+  }
+  const int wco = tid / Cfg::TPC, wt0 = tid % Cfg::TPC;
+  const bool wok = co0 + wco < co_n;
+  const float* wsrc = W + (wok ? (long long)(co0 + wco) * ci_n * 27 : 0LL) + wt0;
+  float vin[Cfg::NIN], vw[Cfg::NW];
+  auto load = [&](int c) {
+    const float* src = inb + c * n;
+#pragma unroll
+    for (int k = 0; k < Cfg::NIN; ++k) vin[k] = valid >> k & 1u ? __ldg(src + off[k]) : 0.f;
+    const float* ws = wsrc + c * 27;
+#pragma unroll
+    for (int k = 0; k < Cfg::NW; ++k) vw[k] = wok && wt0 + k * Cfg::TPC < 27 ? __ldg(ws + k * Cfg::TPC) : 0.f;
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int k = 0; k < Cfg::NIN; ++k) {
+      const int e = tid + k * T;
+      if (e < 3 * IY * IX) s_in[buf][e + e / IX * (IP - IX)] = opnd<BF>(vin[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < Cfg::NW; ++k)
+      if (wt0 + k * Cfg::TPC < 27) s_w[buf][(wt0 + k * Cfg::TPC) * WP + wco] = opnd<BF>(vw[k]);
+  };
+
+  f2 acc[4][4];   // [x voxel][channel pair]
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    const int co = co0 + 8 * cg + 2 * p;
+    const f2 bv = pack2(bias && co < co_n ? __ldg(&bias[co]) : 0.f, bias && co + 1 < co_n ? __ldg(&bias[co + 1]) : 0.f);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) acc[v][p] = bv;
+  }
+  load(0);
+  store(0);
+  __syncthreads();
+  for (int c = 0; c < ci_n; ++c) {
+    const int buf = c & 1;
+    if (c + 1 < ci_n) load(c + 1);
+    const float* xs = s_in[buf] + ty * IP + 4 * tx;
+    const float* ws = s_w[buf] + 8 * cg;
+#pragma unroll
+    for (int dz = 0; dz < 3; ++dz) {
+#pragma unroll
+      for (int dy = 0; dy < 3; ++dy) {
+        const float* row = xs + (dz * IY + dy) * IP;
+        const float4 xa = *reinterpret_cast<const float4*>(row);
+        const float2 xb = *reinterpret_cast<const float2*>(row + 4);
+        const f2 x[6] = {pack2(xa.x, xa.x), pack2(xa.y, xa.y), pack2(xa.z, xa.z),
+                         pack2(xa.w, xa.w), pack2(xb.x, xb.x), pack2(xb.y, xb.y)};
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          const ulonglong2* wp = reinterpret_cast<const ulonglong2*>(ws + (dz * 9 + dy * 3 + dx) * WP);
+          const ulonglong2 w0 = wp[0], w1 = wp[1];
+          const f2 w[4] = {w0.x, w0.y, w1.x, w1.y};
+#pragma unroll
+          for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int v = 0; v < 4; ++v) acc[v][p] = fma2(x[v + dx], w[p], acc[v][p]);
+        }
+      }
+    }
+    if (c + 1 < ci_n) store(buf ^ 1);   // the other buffer: its readers passed the last barrier
+    __syncthreads();
+  }
+  const int gx = x0 + 4 * tx, gy = y0 + ty;
+  if (gy >= ny || gx >= nx) return;
+  float* o = out + (long long)b * out_bs + z * plane + (long long)gy * nx + gx;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    float2 r[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      r[v] = unpack2(acc[v][p]);
+      if (relu) r[v] = make_float2(fmaxf(r[v].x, 0.f), fmaxf(r[v].y, 0.f));
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int co = co0 + 8 * cg + 2 * p + h;
+      if (co >= co_n) continue;
+      const float q[4] = {h ? r[0].y : r[0].x, h ? r[1].y : r[1].x, h ? r[2].y : r[2].x, h ? r[3].y : r[3].x};
+      float* oc = o + co * n;
+      if (vec) {
+        *reinterpret_cast<float4*>(oc) = make_float4(q[0], q[1], q[2], q[3]);
+      } else {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+          if (gx + v < nx) oc[v] = q[v];
+      }
+    }
+  }
+}
+
+template <int CX, int CG, bool BF>
+static cudaError_t launch(const float* in, long long in_bs, int ci, float* out, long long out_bs, int co,
+                          const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz,
+                          cudaStream_t st) {
+  using Cfg = CcCfg<CX, CG>;
+  const int ncb = (co + Cfg::COT - 1) / Cfg::COT;
+  // 16-byte stores: whole groups of four voxels in every row, aligned rows
+  const int vec = nx % 4 == 0 && (uintptr_t)out % 16 == 0 && out_bs % 4 == 0;
+  // grid.z = samples * nz * channel blocks must stay <= 65535: launch sample chunks
+  const int per = std::max(1, 65535 / (nz * ncb));
+  for (int b0 = 0; b0 < B; b0 += per) {
+    const int bc = std::min(per, B - b0);
+    const dim3 grid((nx + CX - 1) / CX, (ny + Cfg::TY - 1) / Cfg::TY, bc * nz * ncb);
+    k_conv3<CX, CG, BF><<<grid, Cfg::THREADS, 0, st>>>(in + (long long)b0 * in_bs, in_bs, ci,
+                                                       out + (long long)b0 * out_bs, out_bs, co, W, bias, relu ? 1 : 0,
+                                                       nx, ny, nz, vec);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+template <int CX, bool BF, typename... A>
+static cudaError_t by_channels(int co, A... a) {
+  return co <= 16 ? launch<CX, 2, BF>(a...) : co <= 32 ? launch<CX, 4, BF>(a...) : launch<CX, 8, BF>(a...);
+}
+
+template <bool BF, typename... A>
+static cudaError_t by_width(int nx, int co, A... a) {
+  if (nx <= 8) return by_channels<8, BF>(co, a...);
+  if ((nx + 15) / 16 % 2) return by_channels<16, BF>(co, a...);   // 32-wide tiles would leave half a tile unused
+  return by_channels<32, BF>(co, a...);
+}
+
+}  // namespace unet_cc
+
+cudaError_t unet_conv3_cc(bool bf, const float* in, long long in_bs, int ci, float* out, long long out_bs, int co,
+                          const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz,
+                          cudaStream_t st) {
+  return bf ? unet_cc::by_width<true>(nx, co, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st)
+            : unet_cc::by_width<false>(nx, co, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st);
+}
+
+}  // namespace clamp
