@@ -1157,7 +1157,86 @@ __global__ void __launch_bounds__(NT) k_gauss3(int nx, int ny, int nz, const flo
   }
 }
 
+// The same stencil for rows of whole, aligned groups of four voxels: a thread owns four x voxels
+// of one (y, 4 x) column and marches along z over `zc` planes.  The x-filtered values of a row
+// serve the three output planes around it (three running sums), so a plane costs three
+// 16-byte loads and six neighbours per four voxels instead of 27 loads and four 64-bit
+// divisions per voxel: 131 -> 24 us at 256x256x128, 57 -> 11 us at 192x192x96 (the volume in and out
+// once: 10 and 4 us of measured HBM).  Terms in the order of k_gauss3 (dz, dy, then x): the same bits.
+__global__ void __launch_bounds__(NT) k_gauss3_z(int nx4, int ny, int nz, int zc, const float* __restrict__ in,
+                                                 float* __restrict__ out, float g0, float g1) {
+  const int idx = blockIdx.x * NT + threadIdx.x;
+  if (idx >= nx4 * ny) return;
+  const int xq = idx % nx4, y = idx / nx4, nx = 4 * nx4;
+  const int z0 = (int)blockIdx.y * zc, z1 = min(z0 + zc, nz);
+  const long long plane = (long long)nx * ny;
+  const float* col = in + (long long)y * nx + 4 * xq;
+  const float wy[3] = {g0, g1, g0};
+  // s[dy][i]: the x-filtered values of rows y - 1 .. y + 1 of plane z (only rows inside are used)
+  float s[3][4];
+  auto filter = [&](int z) {
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy) {
+      const int yy = y + dy - 1;
+      if (yy < 0 || yy >= ny) continue;
+      const float* q = col + z * plane + (dy - 1) * nx;
+      const float4 c = __ldg(reinterpret_cast<const float4*>(q));
+      const float l = xq > 0 ? __ldg(q - 1) : 0.f, r = xq + 1 < nx4 ? __ldg(q + 4) : 0.f;
+      const float v[6] = {l, c.x, c.y, c.z, c.w, r};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        s[dy][i] = g1 * v[i + 1];
+        if (i > 0 || xq > 0) s[dy][i] = fmaf(g0, v[i], s[dy][i]);
+        if (i < 3 || xq + 1 < nx4) s[dy][i] = fmaf(g0, v[i + 2], s[dy][i]);
+      }
+    }
+  };
+  auto add = [&](float (&acc)[4], float wz) {
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy) {
+      const int yy = y + dy - 1;
+      if (yy < 0 || yy >= ny) continue;
+      const float wzy = wz * wy[dy];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] = fmaf(wzy, s[dy][i], acc[i]);
+    }
+  };
+  float cur[4] = {0.f, 0.f, 0.f, 0.f}, nxt[4];   // sums of output planes z and z + 1
+  if (z0 > 0) {
+    filter(z0 - 1);
+    add(cur, g0);
+  }
+  filter(z0);
+  add(cur, g1);
+  for (int z = z0; z < z1; ++z) {
+    // cur holds planes z - 1 and z of output z, s the filtered plane z
+#pragma unroll
+    for (int i = 0; i < 4; ++i) nxt[i] = 0.f;
+    add(nxt, g0);
+    if (z + 1 < nz) {
+      filter(z + 1);
+      add(cur, g0);
+      add(nxt, g1);
+    }
+    *reinterpret_cast<float4*>(out + z * plane + (long long)y * nx + 4 * xq) = make_float4(cur[0], cur[1], cur[2], cur[3]);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cur[i] = nxt[i];
+  }
+}
+
 cudaError_t launch_gauss3(int nx, int ny, int nz, const float* in, float* out, float g0, float g1, cudaStream_t st) {
+  if (nx % 4 == 0 && (uintptr_t)in % 16 == 0 && (uintptr_t)out % 16 == 0 && (long long)nx * ny < (1LL << 30)) {
+    // planes per thread: each march reads two planes more than it writes, so as many (up to 16)
+    // as leave three CTAs per SM
+    const long long cols = ((long long)(nx / 4) * ny + NT - 1) / NT;
+    int zc = 16;
+    while (zc > 1 && cols * ((nz + zc - 1) / zc) < 3 * 152) zc /= 2;
+    const long long zb = (nz + zc - 1) / zc;
+    if (zb <= 65535) {
+      k_gauss3_z<<<dim3((unsigned)cols, (unsigned)zb), NT, 0, st>>>(nx / 4, ny, nz, zc, in, out, g0, g1);
+      return cudaGetLastError();
+    }
+  }
   const long long n = (long long)nx * ny * nz;
   long long b = (n + NT - 1) / NT;
   if (b > 152 * 16) b = 152 * 16;

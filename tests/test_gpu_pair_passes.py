@@ -28,6 +28,19 @@ def _off_by_one(t):
     return v
 
 
+# 27 FMAs of positive terms with weights that sum to 1: 27 x 6e-8 = 1.6e-6 at most
+@pytest.mark.parametrize("shape", [(1, 1, 4), (2, 3, 8), (5, 7, 12), (3, 5, 6), (40, 9, 100), (33, 31, 256), (17, 2, 1024)])
+def test_gauss_matches_oracle(C, shape):
+    x = torch.rand(shape, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+    den = C.Denoiser.gauss(0.8)
+    out, scalar = torch.empty_like(x), torch.empty_like(x)
+    C.denoise(den, x, out)
+    C.denoise(den, _off_by_one(x), scalar)
+    ref = O.denoise_gauss(x.cpu().numpy().astype(np.float64), 0.8)
+    assert np.abs(out.cpu().numpy() - ref).max() < 2e-6
+    assert torch.equal(out, scalar)
+
+
 # one support point at a time through the tables' 32-column words and row blocks: the
 # band-limited and the full-spectrum schedule give the same step
 @pytest.mark.parametrize("nx,ny", [(16, 8), (32, 64), (96, 32), (192, 16), (256, 256)])
