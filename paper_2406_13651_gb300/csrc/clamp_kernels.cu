@@ -804,14 +804,17 @@ __global__ void __launch_bounds__(NT) k_pass_c(Geom g, PassC c) {
   }
 }
 
-// Fused pass C on pairs of adjacent voxels: the same arithmetic as k_pass_c<true, true,
-// false> per voxel, with 16-byte loads of mu and d and 8-byte loads of r and w, so each
-// memory request carries two voxels (n even; the launcher checks the pointers'
-// alignment and otherwise uses the one-voxel kernel).  The look-sum loop keeps the loads
-// of the next two looks in flight and asks L2 for the look six ahead (the grid is small,
-// to keep the Mann loop's re-reads in L2, so each thread needs more bytes in flight).
-constexpr int kPassCPrefetch = 6;   // looks ahead that the look-sum loop prefetches into L2
+// Pass C on pairs of adjacent voxels: the same arithmetic as k_pass_c<PROX, MACE, false> per
+// voxel, with 16-byte loads of mu and d and 8-byte loads of r and w, so each memory request
+// carries two voxels (n even; the launchers check the pointers' alignment and otherwise use
+// the one-voxel kernel).  The look loop keeps the loads of the next two looks in flight and
+// asks L2 for the look six ahead (the grid of the passes with the Mann step is small, to keep its
+// re-reads in L2, so each thread needs more bytes in flight).  The one-voxel kernel had one
+// look's loads in flight: at 192x192x96 with nine looks the MACE step alone took 178 us, now
+// 102 (12 bytes per voxel and row: 57 us of measured HBM), the prox alone 198, now 166 (169 us).
+constexpr int kPassCPrefetch = 6;   // looks ahead that the look loop prefetches into L2
 
+template <bool PROX, bool MACE>
 __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
   const long long n2 = g.n / 2;
   const int L = g.L;
@@ -823,27 +826,33 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
   float4* __restrict__ MUo = reinterpret_cast<float4*>(c.mu);
   const float4* __restrict__ Di = reinterpret_cast<const float4*>(c.d);
   [[maybe_unused]] const long long look_ext = (long long)L * n2, row_ext = (long long)(L + 1) * n2;   // in pairs
-  float acc[2] = {0.f, 0.f};
+  [[maybe_unused]] float acc[2] = {0.f, 0.f};
   for (long long vp = (long long)blockIdx.x * NT + threadIdx.x; vp < n2; vp += (long long)gridDim.x * NT) {
-    CSum wb0, xb0, wb1, xb1;
+    [[maybe_unused]] CSum wb0, xb0, wb1, xb1;
     bool bad = false;
     // two looks ahead in flight: slot a holds look l + 1, slot b look l + 2
     float2 w_n = Wi[vp], r_n = Ri[vp];
-    float4 m_n = __ldcs(&MUi[vp]), d_n = __ldcs(&Di[vp]);
+    float4 m_n = make_float4(0.f, 0.f, 0.f, 0.f), d_n = m_n;
+    if constexpr (PROX) {
+      m_n = __ldcs(&MUi[vp]);
+      d_n = __ldcs(&Di[vp]);
+    }
     float2 w_a = w_n, r_a = r_n;
     float4 m_a = m_n, d_a = d_n;
     if (L > 1) {
       w_a = Wi[n2 + vp];
       r_a = Ri[n2 + vp];
-      m_a = __ldcs(&MUi[n2 + vp]);
-      d_a = __ldcs(&Di[n2 + vp]);
+      if constexpr (PROX) {
+        m_a = __ldcs(&MUi[n2 + vp]);
+        d_a = __ldcs(&Di[n2 + vp]);
+      }
     }
-    float kacc = 0.f;   // sum of K over the looks: non-finite iff some K (so some mu) is
+    [[maybe_unused]] float kacc = 0.f;   // over the looks: non-finite iff some K (so some mu) is
     for (int l = 0; l < L; ++l) {
       const long long i = (long long)l * n2 + vp;
       const float2 wl = w_n, rp = r_n;
-      float4 m = m_n;
-      const float4 dd = d_n;
+      [[maybe_unused]] float4 m = m_n;
+      [[maybe_unused]] const float4 dd = d_n;
       w_n = w_a;
       r_n = r_a;
       m_n = m_a;
@@ -851,77 +860,93 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
       if (l + 2 < L && CLAMP_IN_BOUNDS(i + 2 * n2, look_ext, 201)) {
         w_a = Wi[i + 2 * n2];
         r_a = Ri[i + 2 * n2];
-        m_a = __ldcs(&MUi[i + 2 * n2]);
-        d_a = __ldcs(&Di[i + 2 * n2]);
+        if constexpr (PROX) {
+          m_a = __ldcs(&MUi[i + 2 * n2]);
+          d_a = __ldcs(&Di[i + 2 * n2]);
+        }
       }
       if (l + kPassCPrefetch < L) {   // look l + kPassCPrefetch into L2: no registers held
         const long long ip = i + kPassCPrefetch * n2;
         asm volatile("prefetch.global.L2 [%0];" ::"l"(Wi + ip));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(Ri + ip));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(MUi + ip));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(Di + ip));
+        if constexpr (PROX) {
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(MUi + ip));
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(Di + ip));
+        }
       }
-      if (c.closed_mu) {  // no-aperture ablation: d holds F^H y
-        const float f0 = 1.0f / (1.0f + c.nv / (rp.x + c.nv)), f1 = 1.0f / (1.0f + c.nv / (rp.y + c.nv));
-        m = make_float4(dd.x * f0, dd.y * f0, dd.z * f1, dd.w * f1);
-      } else {
-        const float gm = __ldg(&c.gamma[l]);
-        m = make_float4(fmaf(gm, dd.x, m.x), fmaf(gm, dd.y, m.y), fmaf(gm, dd.z, m.z), fmaf(gm, dd.w, m.w));
+      float2 rn = rp;
+      if constexpr (PROX) {
+        if (c.closed_mu) {  // no-aperture ablation: d holds F^H y
+          const float f0 = 1.0f / (1.0f + c.nv / (rp.x + c.nv)), f1 = 1.0f / (1.0f + c.nv / (rp.y + c.nv));
+          m = make_float4(dd.x * f0, dd.y * f0, dd.z * f1, dd.w * f1);
+        } else {
+          const float gm = __ldg(&c.gamma[l]);
+          m = make_float4(fmaf(gm, dd.x, m.x), fmaf(gm, dd.y, m.y), fmaf(gm, dd.z, m.z), fmaf(gm, dd.w, m.w));
+        }
+        const bool in_look = CLAMP_IN_BOUNDS(i, look_ext, 202);
+        if (in_look) __stcs(&MUo[i], m);   // mu and d are not read again here: evict first
+        const float c0 = c.nv * rp.x * __frcp_rn(fmaf(c.alpha, rp.x, c.nv));
+        const float c1 = c.nv * rp.y * __frcp_rn(fmaf(c.alpha, rp.y, c.nv));
+        const float K0 = c0 + fmaf(m.x, m.x, m.y * m.y), K1 = c1 + fmaf(m.z, m.z, m.w * m.w);
+        rn = make_float2(prox_quad(wl.x, rp.x, K0, c.prox_var, c.inv_prox_var, c.beta, c.inv_beta),
+                         prox_quad(wl.y, rp.y, K1, c.prox_var, c.inv_prox_var, c.beta, c.inv_beta));
+        if (in_look) Ro[i] = rn;
+        // K covers mu: the prox's clip would hide a NaN there.  Without the Mann step's sums below,
+        // products with zero: NaN iff some K or r is not finite
+        if constexpr (MACE) kacc += K0 + K1;
+        else kacc = fmaf(K0, 0.f, fmaf(K1, 0.f, fmaf(rn.x, 0.f, fmaf(rn.y, 0.f, kacc))));
       }
-      const bool in_look = CLAMP_IN_BOUNDS(i, look_ext, 202);
-      if (in_look) __stcs(&MUo[i], m);   // mu and d are not read again here: evict first
-      const float c0 = c.nv * rp.x * __frcp_rn(fmaf(c.alpha, rp.x, c.nv));
-      const float c1 = c.nv * rp.y * __frcp_rn(fmaf(c.alpha, rp.y, c.nv));
-      const float K0 = c0 + fmaf(m.x, m.x, m.y * m.y), K1 = c1 + fmaf(m.z, m.z, m.w * m.w);
-      const float2 rn = make_float2(prox_quad(wl.x, rp.x, K0, c.prox_var, c.inv_prox_var, c.beta, c.inv_beta),
-                                    prox_quad(wl.y, rp.y, K1, c.prox_var, c.inv_prox_var, c.beta, c.inv_beta));
-      if (in_look) Ro[i] = rn;
-      kacc += K0 + K1;   // K covers mu: the prox's clip would hide a NaN there
-      wb0.add(c.ups_look * wl.x);
-      wb1.add(c.ups_look * wl.y);
-      xb0.add(c.ups_look * (2.0f * rn.x - wl.x));
-      xb1.add(c.ups_look * (2.0f * rn.y - wl.y));
+      if constexpr (MACE) {
+        wb0.add(c.ups_look * wl.x);
+        wb1.add(c.ups_look * wl.y);
+        xb0.add(c.ups_look * (2.0f * rn.x - wl.x));
+        xb1.add(c.ups_look * (2.0f * rn.y - wl.y));
+      }
     }
-    const long long ip = (long long)L * n2 + vp;
-    const float2 rpr = Ri[ip], wpr = Wi[ip];
-    wb0.add(c.ups_prior * wpr.x);
-    wb1.add(c.ups_prior * wpr.y);
-    xb0.add(c.ups_prior * (2.0f * rpr.x - wpr.x));
-    xb1.add(c.ups_prior * (2.0f * rpr.y - wpr.y));
-    const float w0 = wb0.get(), w1 = wb1.get(), x0 = xb0.get(), x1 = xb1.get();
-    float num = 0.f;
-    CSum wn0, wn1;
-    float2 rj_n = Ri[vp], wj_n = Wi[vp];
-    float2 rj_a = Ri[n2 + vp], wj_a = Wi[n2 + vp];   // rows 0..L: L + 1 >= 2
-    for (int j = 0; j <= L; ++j) {
-      const long long i = (long long)j * n2 + vp;
-      const float2 rj = rj_n, wj = wj_n;
-      rj_n = rj_a;
-      wj_n = wj_a;
-      if (j + 2 <= L && CLAMP_IN_BOUNDS(i + 2 * n2, row_ext, 203)) {
-        rj_a = Ri[i + 2 * n2];
-        wj_a = Wi[i + 2 * n2];
+    if constexpr (PROX) bad |= !isfinite(kacc);
+    if constexpr (MACE) {
+      const long long ip = (long long)L * n2 + vp;
+      const float2 rpr = Ri[ip], wpr = Wi[ip];
+      wb0.add(c.ups_prior * wpr.x);
+      wb1.add(c.ups_prior * wpr.y);
+      xb0.add(c.ups_prior * (2.0f * rpr.x - wpr.x));
+      xb1.add(c.ups_prior * (2.0f * rpr.y - wpr.y));
+      const float w0 = wb0.get(), w1 = wb1.get(), x0 = xb0.get(), x1 = xb1.get();
+      float num = 0.f;
+      CSum wn0, wn1;
+      float2 rj_n = Ri[vp], wj_n = Wi[vp];
+      float2 rj_a = Ri[n2 + vp], wj_a = Wi[n2 + vp];   // rows 0..L: L + 1 >= 2
+      for (int j = 0; j <= L; ++j) {
+        const long long i = (long long)j * n2 + vp;
+        const float2 rj = rj_n, wj = wj_n;
+        rj_n = rj_a;
+        wj_n = wj_a;
+        if (j + 2 <= L && CLAMP_IN_BOUNDS(i + 2 * n2, row_ext, 203)) {
+          rj_a = Ri[i + 2 * n2];
+          wj_a = Wi[i + 2 * n2];
+        }
+        const float dv0 = rj.x - w0, dv1 = rj.y - w1;
+        num = fmaf(dv0, dv0, fmaf(dv1, dv1, num));
+        const float2 wn = make_float2(fmaf(2.0f * c.rho, x0 - rj.x, wj.x), fmaf(2.0f * c.rho, x1 - rj.y, wj.y));
+        if (CLAMP_IN_BOUNDS(i, row_ext, 204)) Wo[i] = wn;
+        const float ups = j < L ? c.ups_look : c.ups_prior;
+        wn0.add(ups * wn.x);
+        wn1.add(ups * wn.y);
       }
-      const float dv0 = rj.x - w0, dv1 = rj.y - w1;
-      num = fmaf(dv0, dv0, fmaf(dv1, dv1, num));
-      const float2 wn = make_float2(fmaf(2.0f * c.rho, x0 - rj.x, wj.x), fmaf(2.0f * c.rho, x1 - rj.y, wj.y));
-      if (CLAMP_IN_BOUNDS(i, row_ext, 204)) Wo[i] = wn;
-      const float ups = j < L ? c.ups_look : c.ups_prior;
-      wn0.add(ups * wn.x);
-      wn1.add(ups * wn.y);
+      const float wbn0 = wn0.get(), wbn1 = wn1.get();
+      reinterpret_cast<float2*>(c.wbar)[vp] = make_float2(wbn0, wbn1);
+      // a non-finite r, w or K of any look reaches these sums (NaN and Inf propagate through
+      // the adds), so one check per voxel pair replaces one per value
+      bad |= !isfinite(x0) || !isfinite(x1) || !isfinite(w0) || !isfinite(w1) || !isfinite(wbn0) || !isfinite(wbn1);
+      acc[0] += num;
+      acc[1] += (float)(L + 1) * (w0 * w0 + w1 * w1);
     }
-    const float wbn0 = wn0.get(), wbn1 = wn1.get();
-    reinterpret_cast<float2*>(c.wbar)[vp] = make_float2(wbn0, wbn1);
-    // a non-finite r, w or K of any look reaches these sums (NaN and Inf propagate through
-    // the adds), so one check per voxel pair replaces one per value
-    bad = !isfinite(kacc) || !isfinite(x0) || !isfinite(x1) || !isfinite(w0) || !isfinite(w1) ||
-          !isfinite(wbn0) || !isfinite(wbn1);
-    acc[0] += num;
-    acc[1] += (float)(L + 1) * (w0 * w0 + w1 * w1);
     if (bad && c.err) atomicOr(c.err, 1);
   }
-  double* const outs[2] = {c.part_num, c.part_den};
-  block_reduce_store<2>(acc, outs, blockIdx.x);
+  if constexpr (MACE) {
+    double* const outs[2] = {c.part_num, c.part_den};
+    block_reduce_store<2>(acc, outs, blockIdx.x);
+  }
 }
 
 static bool aligned(const void* p, uintptr_t a) { return ((uintptr_t)p % a) == 0; }
@@ -944,22 +969,29 @@ cudaError_t launch_mu_update(const Geom& g, float2* mu, const float2* d, const f
   return cudaGetLastError();
 }
 
+// Pairs of voxels: an even volume and rows that start on the pair's boundary.
+static bool pass_c_pairs(const Geom& g, const PassC& c, bool prox, bool mace) {
+  return g.n % 2 == 0 && aligned(c.w, 8) && aligned(c.r, 8) && (!mace || aligned(c.wbar, 8)) &&
+         (!prox || (aligned(c.mu, 16) && aligned(c.d, 16)));
+}
+
 cudaError_t launch_pass_c_fused(const Geom& g, const PassC& c, cudaStream_t st) {
-  const bool pair = g.n % 2 == 0 && aligned(c.w, 8) && aligned(c.r, 8) && aligned(c.wbar, 8) &&
-                    aligned(c.mu, 16) && aligned(c.d, 16);
   const int nb = passc_fused_blocks(g.n, g.L);
   if (c.exact_prox) k_pass_c<true, true, true><<<nb, NT, 0, st>>>(g, c);
-  else if (pair) k_pass_c_pair<<<nb, NT, 0, st>>>(g, c);
+  else if (pass_c_pairs(g, c, true, true)) k_pass_c_pair<true, true><<<nb, NT, 0, st>>>(g, c);
   else k_pass_c<true, true><<<nb, NT, 0, st>>>(g, c);
   return cudaGetLastError();
 }
 cudaError_t launch_prox_only(const Geom& g, const PassC& c, cudaStream_t st) {
   if (c.exact_prox) k_pass_c<true, false, true><<<passc_blocks(g.n), NT, 0, st>>>(g, c);
+  else if (pass_c_pairs(g, c, true, false)) k_pass_c_pair<true, false><<<passc_blocks(g.n / 2), NT, 0, st>>>(g, c);
   else k_pass_c<true, false><<<passc_blocks(g.n), NT, 0, st>>>(g, c);
   return cudaGetLastError();
 }
+// Every block writes its partial sums: the grid is passc_blocks(n) in either kernel, as the reader expects.
 cudaError_t launch_mace_only(const Geom& g, const PassC& c, cudaStream_t st) {
-  k_pass_c<false, true><<<passc_blocks(g.n), NT, 0, st>>>(g, c);
+  if (pass_c_pairs(g, c, false, true)) k_pass_c_pair<false, true><<<passc_blocks(g.n), NT, 0, st>>>(g, c);
+  else k_pass_c<false, true><<<passc_blocks(g.n), NT, 0, st>>>(g, c);
   return cudaGetLastError();
 }
 

@@ -41,6 +41,33 @@ def test_gauss_matches_oracle(C, shape):
     assert torch.equal(out, scalar)
 
 
+# the same arithmetic per voxel: equal bits.  The convergence error's FP32 partial sums run in
+# another order: at most a few hundred positive terms each, 1e-5 of the sum.
+@pytest.mark.parametrize("L", [1, 2, 3, 9, 17])
+@pytest.mark.parametrize("shape", [(16, 8, 8), (32, 96, 16)])
+def test_pair_passes_match_scalar_passes(C, shape, L):
+    nx, ny, nz = shape
+    wl = I.make_workload("cfg1", seed=5, nx=nx, ny=ny, nz=nz, looks=L, iters=1)
+    p = C.make_params(nx, ny, nz, L, wl.noise_var, 1e-3, max_iters=1)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    y = torch.view_as_complex(torch.randn((L, nz, ny, nx, 2), generator=g, device="cuda"))
+    mu = torch.view_as_complex(torch.randn((L, nz, ny, nx, 2), generator=g, device="cuda"))
+    r = torch.rand((L + 1, nz, ny, nx), generator=g, device="cuda") + 0.05
+    w = torch.rand((L + 1, nz, ny, nx), generator=g, device="cuda") + 0.05
+    pupil, window = torch.from_numpy(wl.pupil).cuda(), torch.from_numpy(wl.window).cuda()
+    got = []
+    for f in (torch.clone, _off_by_one):
+        m, rr, ww, ce = f(mu), f(r), f(w), torch.zeros(1, dtype=torch.float64, device="cuda")
+        wbar = f(r[0])
+        C.forward_prox(p, 3, y, pupil, window, m, rr, ww)
+        C.mace_step(p, rr, ww, wbar, ce)
+        got.append((m, rr, ww, wbar, float(ce.item())))
+    for a, b in zip(got[0][:4], got[1][:4]):
+        assert torch.isfinite(torch.view_as_real(a) if a.is_complex() else a).all()
+        assert torch.equal(a, b)
+    assert abs(got[0][4] - got[1][4]) <= 1e-5 * got[1][4]
+
+
 # one support point at a time through the tables' 32-column words and row blocks: the
 # band-limited and the full-spectrum schedule give the same step
 @pytest.mark.parametrize("nx,ny", [(16, 8), (32, 64), (96, 32), (192, 16), (256, 256)])
