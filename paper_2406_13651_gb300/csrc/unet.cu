@@ -561,73 +561,127 @@ static cudaError_t tconv_dgrad(const float* dout, long long dout_bs, int co, flo
   return cudaGetLastError();
 }
 
-// dW[ci][co][d] += sum_{b, v} in[b][ci][v] dout[b][co][2v + d].  A CTA takes 16 input and 4
-// output channels (16 x 4 x 8 sums, two per thread: d pairs of one (ci, co)) and a share of the
-// 64-voxel runs of (sample, z, y) rows; each run's inputs and children are staged once in
-// shared memory, so global memory is read once per channel block instead of once per
-// (ci, co) pair.  FP32 sums, one atomic per sum and CTA.
-constexpr int TW_CI = 16, TW_CO = 4, TW_V = 64;
-__global__ void __launch_bounds__(UT) k_tconv_wgrad(const float* __restrict__ in, int ci_n,
-                                                    const float* __restrict__ dout, long long dout_bs, int co_n,
-                                                    float* __restrict__ dW, int B, int nx, int ny, int nz, int bf) {
-  __shared__ float s_x[TW_CI][TW_V + 1];
-  __shared__ __align__(16) float s_g[TW_CO * 4][2 * TW_V + 2];   // rows (co, dz, dy) of 2 TW_V children
-  const int ix = nx / 2, iy = ny / 2, iz = nz / 2;
-  const long long n = (long long)nx * ny * nz, in_n = n / 8, iplane = (long long)ix * iy;
+// dW[ci][co][d] += sum_{b, v} in[b][ci][v] dout[b][co][2v + d]: a product of a [ci][voxel] and a
+// [voxel][(co, d)] matrix.  A CTA takes 32 input and 16 output channels (32 x 128 sums, 8 x 4 per
+// thread, so three 16-byte shared loads feed 32 FMAs) and a share of the 32-voxel chunks of
+// the samples' flat voxel order, whatever the rows' width; the next chunk's loads are in
+// flight in registers while the current one's FMAs run.  Bound by FMA issue (24 x 64x64x32,
+// 32 -> 16: 43 us of FMAs, 30 us of HBM).  Two sums per thread walked 64-voxel rows, mostly
+// padding at the coarse levels (16 wide: a quarter used): 807 us there and 765 us for 64 -> 32 at
+// half size, now 124 and 63.  A chain is 256 voxels; each is added in FP32 to a second
+// register sum, those with one atomic per sum and CTA.
+constexpr int TW_CI = 32, TW_CO = 16, TW_V = 32, TW_NT = 128, TW_CHAIN = 8;   // TW_CHAIN: chunks per chain
+constexpr int TW_XP = TW_CI + 4, TW_GP = TW_CO * 8 + 8;                       // row pitches (floats)
+__global__ void __launch_bounds__(TW_NT, 3) k_tconv_wgrad(const float* __restrict__ in, int ci_n,
+                                                          const float* __restrict__ dout, long long dout_bs, int co_n,
+                                                          float* __restrict__ dW, int B, int nx, int ny, int nz, int bf) {
+  __shared__ __align__(16) float s_x[2][TW_V][TW_XP];   // [voxel][ci]
+  __shared__ __align__(16) float s_g[2][TW_V][TW_GP];   // [voxel][co][d]
+  const int ix = nx / 2, iy = ny / 2, iz = nz / 2, in_n = ix * iy * iz;
+  const long long plane = (long long)nx * ny, n = plane * nz;
   const int ci0 = blockIdx.y * TW_CI, co0 = blockIdx.z * TW_CO;
-  const int runs_x = (ix + TW_V - 1) / TW_V;
-  const long long runs = (long long)B * iz * iy * runs_x;
-  const int ci = threadIdx.x / 16, co = (threadIdx.x / 4) % 4, zy = threadIdx.x % 4;
-  float a0 = 0.f, a1 = 0.f;
-  for (long long r = blockIdx.x; r < runs; r += gridDim.x) {
-    const int x0 = (int)(r % runs_x) * TW_V;
-    long long t = r / runs_x;
-    const int y = (int)(t % iy);
-    t /= iy;
-    const int z = (int)(t % iz);
-    const long long b = t / iz;
-    const int w = min(TW_V, ix - x0);
-    __syncthreads();
-    for (int e = threadIdx.x; e < TW_CI * TW_V; e += UT) {
-      const int c = e / TW_V, x = e % TW_V;
-      s_x[c][x] = ci0 + c < ci_n && x < w
-                      ? opr(__ldg(&in[(b * ci_n + ci0 + c) * in_n + z * iplane + (long long)y * ix + x0 + x]), bf)
-                      : 0.f;
+  const int per_b = (in_n + TW_V - 1) / TW_V;
+  const long long chunks = (long long)B * per_b;
+  const long long c_begin = chunks * blockIdx.x / gridDim.x, c_end = chunks * (blockIdx.x + 1) / gridDim.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int XT = TW_V * TW_CI / TW_NT;              // inputs staged per thread: voxel `lane`, channel warp + 4 k
+  constexpr int GT = TW_V * TW_CO * 4 / TW_NT;          // children pairs per thread
+  // pair k: voxel lane / 4 + 8 (k % 4), row (co, dz, dy) = lane % 4 + 4 warp + 16 (k / 4)
+  const int gv0 = lane >> 2, gr0 = (lane & 3) + 4 * warp;
+  float xv[XT];
+  float2 gv[GT];
+  auto load = [&](long long c) {
+    const int b = (int)(c / per_b), v0 = (int)(c % per_b) * TW_V;
+    const float* xs = in + ((long long)b * ci_n + ci0) * in_n + v0 + lane;
+#pragma unroll
+    for (int k = 0; k < XT; ++k) {
+      const int ci = warp + 4 * k;
+      xv[k] = v0 + lane < in_n && ci0 + ci < ci_n ? __ldg(xs + (long long)ci * in_n) : 0.f;
     }
-    for (int e = threadIdx.x; e < TW_CO * 4 * 2 * TW_V; e += UT) {
-      const int x = e % (2 * TW_V), row = e / (2 * TW_V), c = row / 4, d = row % 4;
-      s_g[row][x] = co0 + c < co_n && x < 2 * w
-                        ? opr(__ldg(&dout[b * dout_bs + (long long)(co0 + c) * n + (long long)(2 * z + (d >> 1)) * nx * ny +
-                                          (long long)(2 * y + (d & 1)) * nx + 2 * x0 + x]), bf)
-                        : 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int v = v0 + gv0 + 8 * j;
+      const int x = v % ix, y = v / ix % iy, z = v / (ix * iy);
+      const float* gs = dout + b * dout_bs + (long long)(2 * z) * plane + (long long)(2 * y) * nx + 2 * x;
+#pragma unroll
+      for (int i = 0; i < GT / 4; ++i) {
+        const int row = gr0 + 16 * i, co = co0 + row / 4;
+        gv[4 * i + j] = v < in_n && co < co_n
+                            ? __ldg(reinterpret_cast<const float2*>(gs + co * n + ((row >> 1) & 1) * plane + (row & 1) * nx))
+                            : make_float2(0.f, 0.f);
+      }
     }
-    __syncthreads();
-    const float* gp = s_g[co * 4 + zy];
-    const float* xp = s_x[ci];
-    float r0 = 0.f, r1 = 0.f;   // a run's sums apart: short FP32 chains
-#pragma unroll 8
-    for (int x = 0; x < TW_V; ++x) {
-      const float xv = xp[x];
-      const float2 g = *reinterpret_cast<const float2*>(gp + 2 * x);
-      r0 = fmaf(xv, g.x, r0);
-      r1 = fmaf(xv, g.y, r1);
-    }
-    a0 += r0;
-    a1 += r1;
+  };
+  auto store = [&](int buf) {
+#pragma unroll
+    for (int k = 0; k < XT; ++k) s_x[buf][lane][warp + 4 * k] = opr(xv[k], bf);
+#pragma unroll
+    for (int k = 0; k < GT; ++k)
+      *reinterpret_cast<float2*>(&s_g[buf][gv0 + 8 * (k % 4)][2 * (gr0 + 16 * (k / 4))]) =
+          make_float2(opr(gv[k].x, bf), opr(gv[k].y, bf));
+  };
+  float acc[8][4], sum[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = sum[i][j] = 0.f;
+  auto flush = [&]() {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        sum[i][j] += acc[i][j];
+        acc[i][j] = 0.f;
+      }
+  };
+  if (c_begin < c_end) {
+    load(c_begin);
+    store(0);
   }
-  if (ci0 + ci < ci_n && co0 + co < co_n) {
-    float* d = &dW[((long long)(ci0 + ci) * co_n + co0 + co) * 8 + 2 * zy];
-    atomicAdd(d, a0);
-    atomicAdd(d + 1, a1);
+  __syncthreads();
+  for (long long c = c_begin; c < c_end; ++c) {
+    const int buf = (int)(c - c_begin) & 1;
+    if (c + 1 < c_end) load(c + 1);
+    const float* xp = &s_x[buf][0][8 * warp];
+    const float* gp = &s_g[buf][0][4 * lane];
+#pragma unroll 4
+    for (int v = 0; v < TW_V; ++v) {
+      const float4 xa = *reinterpret_cast<const float4*>(xp + v * TW_XP);
+      const float4 xb = *reinterpret_cast<const float4*>(xp + v * TW_XP + 4);
+      const float4 g = *reinterpret_cast<const float4*>(gp + v * TW_GP);
+      const float x[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        acc[i][0] = fmaf(x[i], g.x, acc[i][0]);
+        acc[i][1] = fmaf(x[i], g.y, acc[i][1]);
+        acc[i][2] = fmaf(x[i], g.z, acc[i][2]);
+        acc[i][3] = fmaf(x[i], g.w, acc[i][3]);
+      }
+    }
+    if ((c - c_begin) % TW_CHAIN == TW_CHAIN - 1) flush();
+    if (c + 1 < c_end) store(buf ^ 1);   // the other buffer: its readers passed the last barrier
+    __syncthreads();
+  }
+  flush();
+  const int co = co0 + lane / 2;
+  if (co >= co_n) return;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int ci = ci0 + 8 * warp + i;
+    if (ci >= ci_n) continue;
+    float* d = dW + ((long long)ci * co_n + co) * 8 + 4 * (lane & 1);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) atomicAdd(d + j, sum[i][j]);
   }
 }
 
 static cudaError_t tconv_wgrad(const float* in, int ci, const float* dout, long long dout_bs, int co, float* dW, int B,
                                int nx, int ny, int nz, int bf, cudaStream_t st) {
   const int bi = (ci + TW_CI - 1) / TW_CI, bo = (co + TW_CO - 1) / TW_CO;
-  const long long runs = (long long)B * (nz / 2) * (ny / 2) * ((nx / 2 + TW_V - 1) / TW_V);
-  const long long per = std::max(1, 152 * 8 / (bi * bo));
-  k_tconv_wgrad<<<dim3((unsigned)std::min(runs, per), bi, bo), UT, 0, st>>>(in, ci, dout, dout_bs, co, dW, B, nx, ny, nz, bf);
+  const long long chunks = (long long)B * (((long long)nx * ny * nz / 8 + TW_V - 1) / TW_V);
+  const long long per = std::max(1, 152 * 3 / (bi * bo));   // one wave of three CTAs per SM
+  k_tconv_wgrad<<<dim3((unsigned)std::min(chunks, per), bi, bo), TW_NT, 0, st>>>(in, ci, dout, dout_bs, co, dW, B, nx, ny,
+                                                                                 nz, bf);
   return cudaGetLastError();
 }
 
