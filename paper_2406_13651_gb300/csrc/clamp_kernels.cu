@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(NT) k_ab_z(Geom g, AgentScalars s, const float
 
 // ---------------------------------------------------------------- generic single-transform passes
 
-enum RowMode { ROW_PLAIN = 0, ROW_SIM = 1, ROW_ADJ = 2, ROW_BX = 3 };
+enum RowMode { ROW_PLAIN = 0, ROW_SIM = 1, ROW_BX = 3 };
 enum ColMode { COL_PLAIN = 0, COL_SIM = 1, COL_ADJ = 2 };
 
 struct RowArgs {
@@ -257,7 +257,7 @@ struct RowArgs {
   float2* out;
   const float* rvol;   // ROW_SIM: reflectance [n]
   const float* rprev;  // ROW_BX: r' [L][n]
-  float scale;         // 1/sqrt(N) (times mu_scale for ROW_ADJ)
+  float scale;         // 1/sqrt(N) (times mu_scale in the adjoint)
   float floor;         // ROW_BX: sigma_w^2 / alpha
   double* s3;          // ROW_BX partials
   int px;              // ROW_BX partials per look
@@ -265,8 +265,76 @@ struct RowArgs {
   int nx;
 };
 
-template <int N, bool INV, int MODE, int V = 0>
-__global__ void __launch_bounds__(NT) k_row(RowArgs a, const float2* __restrict__ tw) {
+// Launch variant 0: a row's threads hold its points in registers and exchange them once through
+// shared memory (fft_reg.cuh), each row within one warp, where the tile version (variants 1 and
+// 2) stages the tile and passes it through shared memory, with a block barrier, at every
+// stage.  Set-up of 128^3, nine looks: rows 51 -> 43 us, columns 74 -> 44 (y) and 92 -> 49 (z; 45 us
+// of measured HBM each); 64x64x32, 32 looks: 122 -> 75 us for the six.
+template <int N, bool INV, int MODE>
+__global__ void __launch_bounds__(NT, 2) k_row_reg(RowArgs a, const float2* __restrict__ twA, const float2* __restrict__ twB) {
+  constexpr int R1 = RRow<N>::R1, R2 = RRow<N>::R2, T = RRow<N>::T, LINES = NT / T;
+  static_assert(LINES == rows_per_cta(N), "rows per CTA");
+  const int line = threadIdx.x / T, j = threadIdx.x % T;
+  float2* sl = reinterpret_cast<float2*>(dyn_smem) + line * RRow<N>::LS;
+  const long long row = (long long)blockIdx.x * LINES + line, e0 = row * N;
+  float acc[1] = {0.f};
+  if constexpr (INV) {
+    static_assert(MODE == ROW_PLAIN || MODE == ROW_BX, "inverse rows");
+    float rpv[R2];
+    if constexpr (MODE == ROW_BX) {
+#pragma unroll
+      for (int r = 0; r < R2; ++r) rpv[r] = a.rprev[e0 + j + r * R1];
+    }
+#pragma unroll
+    for (int i = 0; i < RRow<N>::NB; ++i) {
+      const int b = j + i * T;
+      if (R2 % T != 0 && b >= R2) continue;
+      float2 v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) v[r] = a.in[e0 + b + r * R2];
+      rrow_inv_outer<N>(v, sl, b);
+    }
+    __syncwarp();
+    float2 u[R2];
+    rrow_inv_mid<N>(u, sl, j, twA);
+#pragma unroll
+    for (int r = 0; r < R2; ++r) {
+      const float2 v = cscale(u[r], a.scale);
+      if constexpr (MODE == ROW_BX) acc[0] += cabs2(v) / (rpv[r] + a.floor);
+      a.out[e0 + j + r * R1] = v;
+    }
+  } else {
+    static_assert(MODE == ROW_PLAIN || MODE == ROW_SIM, "forward rows");
+    float2 u[R2];
+#pragma unroll
+    for (int r = 0; r < R2; ++r) u[r] = a.in[e0 + j + r * R1];
+    if constexpr (MODE == ROW_SIM) {
+      const float* rv = a.rvol + e0 % a.n + j;   // a row lies in one look
+#pragma unroll
+      for (int r = 0; r < R2; ++r) u[r] = cscale(u[r], sqrtf(rv[r * R1]));
+    }
+    rrow_fwd_mid<N>(u, sl, j);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < RRow<N>::NB; ++i) {
+      const int b = j + i * T;
+      if (R2 % T != 0 && b >= R2) continue;
+      float2 v[R1];
+      rrow_fwd_outer<N>(v, sl, b, twB);
+#pragma unroll
+      for (int r = 0; r < R1; ++r) a.out[e0 + b + r * R2] = cscale(v[r], a.scale);
+    }
+  }
+  if constexpr (MODE == ROW_BX) {
+    double* const outs[1] = {a.s3};
+    const long long first = (long long)blockIdx.x * LINES * N, look = first / a.n;
+    block_reduce_store<1>(acc, outs, look * a.px + (blockIdx.x - look * (a.n / ((long long)LINES * N))));
+  }
+}
+
+// Launch variants 1 and 2 of the full-spectrum schedule's inverse row pass: tiles in shared memory.
+template <int N, int V>
+__global__ void __launch_bounds__(NT) k_row_bx(RowArgs a, const float2* __restrict__ tw) {
   constexpr int LX = variant_rows(N, V), LD = N + 1;
   using PL = std::conditional_t<V == 1, PlanB<N>, Plan<N>>;
   float2* sm = reinterpret_cast<float2*>(dyn_smem);
@@ -283,24 +351,17 @@ __global__ void __launch_bounds__(NT) k_row(RowArgs a, const float2* __restrict_
     const int e = threadIdx.x + p * NT;
     if (CNT % NT == 0 || e < CNT) {
       const int line = e / N, i = e - line * N;
-      float2 v = iv[p];
-      if constexpr (MODE == ROW_SIM) {
-        const long long vox = (e0 + e) % a.n;
-        v = cscale(v, sqrtf(a.rvol[vox]));
-      }
-      sm[line * LD + i] = v;
+      sm[line * LD + i] = iv[p];
     }
   }
   __syncthreads();
-  fft_tile<N, LX, NT, INV, PL>(sm, tw);
+  fft_tile<N, LX, NT, true, PL>(sm, tw);
   float acc[1] = {0.f};
   float rpv[PER];
-  if constexpr (MODE == ROW_BX) {
 #pragma unroll
-    for (int p = 0; p < PER; ++p) {
-      const int e = threadIdx.x + p * NT;
-      if (CNT % NT == 0 || e < CNT) rpv[p] = a.rprev[e0 + e];
-    }
+  for (int p = 0; p < PER; ++p) {
+    const int e = threadIdx.x + p * NT;
+    if (CNT % NT == 0 || e < CNT) rpv[p] = a.rprev[e0 + e];
   }
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
@@ -308,16 +369,14 @@ __global__ void __launch_bounds__(NT) k_row(RowArgs a, const float2* __restrict_
     if (CNT % NT == 0 || e < CNT) {
       const int line = e / N, i = e - line * N;
       const float2 v = cscale(sm[line * LD + i], a.scale);
-      if constexpr (MODE == ROW_BX) acc[0] += cabs2(v) / (rpv[p] + a.floor);
+      acc[0] += cabs2(v) / (rpv[p] + a.floor);
       a.out[e0 + e] = v;
     }
   }
-  if constexpr (MODE == ROW_BX) {
-    double* const outs[1] = {a.s3};
-    const long long look = e0 / a.n;
-    const long long bpl = a.n / ((long long)LX * N);
-    block_reduce_store<1>(acc, outs, look * a.px + (blockIdx.x - look * bpl));
-  }
+  double* const outs[1] = {a.s3};
+  const long long look = e0 / a.n;
+  const long long bpl = a.n / ((long long)LX * N);
+  block_reduce_store<1>(acc, outs, look * a.px + (blockIdx.x - look * bpl));
 }
 
 struct ColArgs {
@@ -335,8 +394,50 @@ struct ColArgs {
   int zaxis;           // 1 when the FFT axis is z (aperture epilogue / prologue)
 };
 
-template <int N, bool INV, int MODE, int V = 0>
-__global__ void __launch_bounds__(NT) k_col(ColArgs a, const float2* __restrict__ tw) {
+// Launch variant 0: 16 adjacent lines per CTA, points in registers, one exchange (fft_reg.cuh).
+template <int N, bool INV, int MODE>
+__global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_col_reg(ColArgs a, const float2* __restrict__ twB) {
+  constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2, NB = RCol<N>::NB;
+  float2* sm = reinterpret_cast<float2*>(dyn_smem);
+  const int col = threadIdx.x % RCOLS, j = threadIdx.x / RCOLS;
+  const int x = blockIdx.x * RCOLS + col, fixed = blockIdx.y, l = blockIdx.z;
+  const long long base = (long long)l * a.n + (long long)fixed * a.slab + x;
+  [[maybe_unused]] const float pup = MODE == COL_PLAIN ? 0.f : __ldg(&a.pupil[fixed * a.nx + x]);   // z axis, fixed = ky
+  float2 u[R2];
+#pragma unroll
+  for (int r = 0; r < R2; ++r) u[r] = a.in[base + (j + r * R1) * a.stride];
+  if constexpr (MODE == COL_ADJ) {
+#pragma unroll
+    for (int r = 0; r < R2; ++r) u[r] = cscale(u[r], pup * __ldg(&a.window[j + r * R1]));
+  }
+  rcol_first<N, INV>(u, sm, col, j);
+#pragma unroll
+  for (int i = 0; i < NB; ++i) {
+    const int b = j + i * R1;
+    if (R2 % R1 != 0 && b >= R2) continue;
+    [[maybe_unused]] float2 et[R1];
+    if constexpr (MODE == COL_SIM) {   // in flight during the second stage
+#pragma unroll
+      for (int r = 0; r < R1; ++r) et[r] = a.eta[base + (b + r * R2) * a.stride];
+    }
+    float2 v[R1];
+    rcol_second<N, INV>(v, sm, col, b, twB);
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const int k = b + r * R2;
+      float2 o = cscale(v[r], a.scale);
+      if constexpr (MODE == COL_SIM) {   // y = a v + sigma_w eta
+        const float av = pup * __ldg(&a.window[k]);
+        o = make_float2(fmaf(av, o.x, a.sig_w * et[r].x), fmaf(av, o.y, a.sig_w * et[r].y));
+      }
+      a.out[base + k * a.stride] = o;
+    }
+  }
+}
+
+// Launch variants 1 and 2 of the full-spectrum schedule's inverse y pass: tiles in shared memory.
+template <int N, int V>
+__global__ void __launch_bounds__(NT) k_col_by(ColArgs a, const float2* __restrict__ tw) {
   constexpr int LD = N + 1, LCV = variant_cols(V);
   using PL = std::conditional_t<V == 1, PlanB<N>, Plan<N>>;
   float2* sm = reinterpret_cast<float2*>(dyn_smem);
@@ -352,30 +453,16 @@ __global__ void __launch_bounds__(NT) k_col(ColArgs a, const float2* __restrict_
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
     const int e = threadIdx.x + p * NT;
-    if (CNT % NT == 0 || e < CNT) {
-      const int line = e % LCV, i = e / LCV;
-      float2 v = iv[p];
-      if constexpr (MODE == COL_ADJ) {  // z axis, fixed = ky
-        v = cscale(v, __ldg(&a.pupil[fixed * a.nx + x0 + line]) * __ldg(&a.window[i]));
-      }
-      sm[line * LD + i] = v;
-    }
+    if (CNT % NT == 0 || e < CNT) sm[e % LCV * LD + e / LCV] = iv[p];
   }
   __syncthreads();
-  fft_tile<N, LCV, NT, INV, PL>(sm, tw);
+  fft_tile<N, LCV, NT, true, PL>(sm, tw);
 #pragma unroll
   for (int p = 0; p < PER; ++p) {
     const int e = threadIdx.x + p * NT;
     if (!(CNT % NT == 0 || e < CNT)) continue;
     const int line = e % LCV, i = e / LCV;
-    float2 v = cscale(sm[line * LD + i], a.scale);
-    const long long gi = base + i * a.stride + line;
-    if constexpr (MODE == COL_SIM) {  // z axis, fixed = ky: y = a v + sigma_w eta
-      const float av = __ldg(&a.pupil[fixed * a.nx + x0 + line]) * __ldg(&a.window[i]);
-      const float2 et = a.eta[gi];
-      v = make_float2(fmaf(av, v.x, a.sig_w * et.x), fmaf(av, v.y, a.sig_w * et.y));
-    }
-    a.out[gi] = v;
+    a.out[base + i * a.stride + line] = cscale(sm[line * LD + i], a.scale);
   }
 }
 
@@ -398,25 +485,39 @@ static cudaError_t dispatch_len(int N, F&& f) {
 
 template <int N, bool INV, int MODE, int V = 0>
 static cudaError_t run_row(const Geom& g, const RowArgs& a, cudaStream_t st) {
-  constexpr int LX = variant_rows(N, V);
-  const size_t smem = (size_t)LX * (N + 1) * sizeof(float2);
-  auto kern = k_row<N, INV, MODE, V>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const long long rows = (long long)g.L * g.nz * g.ny;
-  kern<<<(unsigned)(rows / LX), NT, smem, st>>>(a, tw_ptr(N));
+  if constexpr (N < 16) {   // nx is a multiple of 16
+    return cudaErrorInvalidValue;
+  } else if constexpr (V == 0) {
+    constexpr size_t smem = (size_t)rows_per_cta(N) * RRow<N>::LS * sizeof(float2);
+    static_assert(smem <= 48 * 1024, "default shared-memory limit");
+    k_row_reg<N, INV, MODE><<<(unsigned)(rows / rows_per_cta(N)), NT, smem, st>>>(a, twiddle_table_a(N), twiddle_table_b(N));
+  } else {
+    static_assert(INV && MODE == ROW_BX, "tile variants");
+    constexpr int LX = variant_rows(N, V);
+    const size_t smem = (size_t)LX * (N + 1) * sizeof(float2);
+    auto kern = k_row_bx<N, V>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)(rows / LX), NT, smem, st>>>(a, tw_ptr(N));
+  }
   return cudaGetLastError();
 }
 
 template <int N, bool INV, int MODE, int V = 0>
 static cudaError_t run_col(const Geom& g, const ColArgs& a, int fixed_count, cudaStream_t st) {
-  constexpr int LCV = variant_cols(V);
-  const size_t smem = (size_t)LCV * (N + 1) * sizeof(float2);
-  auto kern = k_col<N, INV, MODE, V>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(g.nx / LCV, fixed_count, g.L);
-  kern<<<grid, NT, smem, st>>>(a, tw_ptr(N));
+  if constexpr (V == 0) {
+    static_assert(RCol<N>::SMEM <= 48 * 1024, "default shared-memory limit");
+    k_col_reg<N, INV, MODE><<<dim3(g.nx / RCOLS, fixed_count, g.L), RCol<N>::THREADS, RCol<N>::SMEM, st>>>(a, twiddle_table_b(N));
+  } else {
+    static_assert(INV && MODE == COL_PLAIN, "tile variants");
+    constexpr int LCV = variant_cols(V);
+    const size_t smem = (size_t)LCV * (N + 1) * sizeof(float2);
+    auto kern = k_col_by<N, V>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3(g.nx / LCV, fixed_count, g.L), NT, smem, st>>>(a, tw_ptr(N));
+  }
   return cudaGetLastError();
 }
 
