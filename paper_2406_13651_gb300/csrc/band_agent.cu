@@ -18,7 +18,7 @@
 //                      S1 = ||d||^2, S3 = sum D |d|^2;  forward x-FFT of d, kept on B
 //   P4 y pass on B   : forward y-FFT, kept on S                         -> [z][S]
 //   P5 z pass on S   : forward z-FFT -> F d on S;  S2 = ||a F d||^2
-// then gamma = S1 / (S2 / sigma_w^2 + S3) and the elementwise pass C.  Only P3 touches
+// whose last CTA per look forms gamma = S1 / (S2 / sigma_w^2 + S3); then the elementwise pass C.  Only P3 touches
 // every voxel: it reads mu, r' and writes d, plus two band rows.
 #include "clamp_kernels.cuh"
 #include "fft_reg.cuh"
@@ -207,6 +207,7 @@ __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_inv(
       if (CLAMP_IN_BOUNDS(fi, sL, 105)) a.Fd[fi] = cscale(v[r], a.sc_z);   // Gz, in place
     }
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *reinterpret_cast<unsigned*>(&a.mures[l]) = 0u;   // look_step's count
   double* const outs[1] = {a.s4};
   block_sums<RCol<N>::THREADS, 1>(acc, outs, (long long)l * gridDim.x + blockIdx.x);
 }
@@ -357,7 +358,49 @@ __global__ void __launch_bounds__(RowCta<N, V>::THREADS, RowCta<N, V>::MINB)
 
 // ---------------------------------------------------------------- P5: z pass on the support (forward)
 
-// BAND_GRAD: F d on the support (in place) and S2 = ||a F d||^2.  BAND_SPEC: writes M.
+// gamma_l = S1 / (S2 / sigma_w^2 + S3) and the floored mu-residual sqrt(S1) / (sqrt(S4) / sigma_w^2) from
+// the look's partial sums: by the last of the look's CTAs of the forward z pass (a kernel of its
+// own cost a launch and 7 us on a small scene, where the passes are a chain of such latencies).
+// The CTAs are counted in the look's mu-residual slot, which k_band_z_inv zeroes.
+template <int NTH>
+__device__ __forceinline__ void look_step(const BandArgs& a, int l, int pS) {
+  constexpr int NW = (NTH + 31) / 32;
+  __shared__ bool s_last;
+  __shared__ double red[NW][4];
+  unsigned* ticket = reinterpret_cast<unsigned*>(&a.mures[l]);
+  if (threadIdx.x == 0) {   // this thread wrote the CTA's partial sum
+    __threadfence();
+    s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double v[4] = {0, 0, 0, 0};
+  for (int i = threadIdx.x; i < a.px; i += NTH) {
+    v[0] += __ldcg(&a.s1[(long long)l * a.px + i]);
+    v[2] += __ldcg(&a.s3[(long long)l * a.px + i]);
+  }
+  for (int i = threadIdx.x; i < pS; i += NTH) {
+    v[1] += __ldcg(&a.s2[(long long)l * pS + i]);
+    v[3] += __ldcg(&a.s4[(long long)l * pS + i]);
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v[k];
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double S[4] = {0, 0, 0, 0};
+  for (int w = 0; w < NW; ++w)
+    for (int k = 0; k < 4; ++k) S[k] += red[w][k];
+  const double den = S[1] / (double)a.nv + S[2];
+  a.gamma[l] = den > 0 ? (float)(S[0] / den) : 0.0f;
+  a.mures[l] = S[3] > 0 ? sqrt(S[0]) / (sqrt(S[3]) / (double)a.nv) : 0.0;
+}
+
+// BAND_GRAD: F d on the support (in place), S2 = ||a F d||^2 and the look's step.  BAND_SPEC: writes M.
 template <int N, int MODE>
 __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_fwd(BandArgs a, const float2* __restrict__ twB) {
   [[maybe_unused]] const long long sL = (long long)a.L * a.nz * a.t.nSp;   // buffer extent
@@ -398,37 +441,7 @@ __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_fwd(
   if constexpr (MODE == BAND_GRAD) {
     double* const outs[1] = {a.s2};
     block_sums<RCol<N>::THREADS, 1>(acc, outs, (long long)l * gridDim.x + blockIdx.x);
-  }
-}
-
-// gamma_l = S1 / (S2 / sigma_w^2 + S3) and the floored mu-residual sqrt(S1) / (sqrt(S4) / sigma_w^2).
-__global__ void __launch_bounds__(NT) k_band_gamma(BandArgs a, int pS, float nv, float* gamma, double* mures) {
-  const int l = blockIdx.x;
-  __shared__ double red[NT][4];
-  double v1 = 0, v2 = 0, v3 = 0, v4 = 0;
-  for (int i = threadIdx.x; i < a.px; i += NT) {
-    v1 += a.s1[(long long)l * a.px + i];
-    v3 += a.s3[(long long)l * a.px + i];
-  }
-  for (int i = threadIdx.x; i < pS; i += NT) {
-    v2 += a.s2[(long long)l * pS + i];
-    v4 += a.s4[(long long)l * pS + i];
-  }
-  red[threadIdx.x][0] = v1;
-  red[threadIdx.x][1] = v2;
-  red[threadIdx.x][2] = v3;
-  red[threadIdx.x][3] = v4;
-  __syncthreads();
-  for (int o = NT / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o)
-      for (int k = 0; k < 4; ++k) red[threadIdx.x][k] += red[threadIdx.x + o][k];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const double S1 = red[0][0], S2 = red[0][1], S3 = red[0][2], S4 = red[0][3];
-    const double den = S2 / (double)nv + S3;
-    gamma[l] = den > 0 ? (float)(S1 / den) : 0.0f;
-    mures[l] = S4 > 0 ? sqrt(S1) / (sqrt(S4) / (double)nv) : 0.0;
+    look_step<RCol<N>::THREADS>(a, l, gridDim.x);
   }
 }
 
@@ -569,13 +582,14 @@ cudaError_t launch_band_agent(const BandArgs& a, int L, float nv, float* gamma, 
   BandArgs b = a;
   b.L = L;
   b.px = band_px(a.nx, a.ny, a.nz, x_variant);
+  b.nv = nv;
+  b.gamma = gamma;
+  b.mures = mures;
   BAND_TRY(run_z(b, L, true, BAND_GRAD, st));
   BAND_TRY(run_y(b, L, true, st));
   BAND_TRY(run_x(b, L, BAND_GRAD, x_variant, st));
   BAND_TRY(run_y(b, L, false, st));
-  BAND_TRY(run_z(b, L, false, BAND_GRAD, st));
-  k_band_gamma<<<L, NT, 0, st>>>(b, band_pS(BandShape{a.t.nS, a.t.nSp, a.t.nbx, a.t.nbxp}), nv, gamma, mures);
-  return cudaGetLastError();
+  return run_z(b, L, false, BAND_GRAD, st);
 }
 
 cudaError_t bounds_site_band(unsigned int* site, bool reset) { return bounds_site_local(site, reset); }

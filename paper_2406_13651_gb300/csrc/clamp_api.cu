@@ -841,7 +841,6 @@ static clamp_status iterate_impl(const clamp_params* p, const Derived& d, int k_
     } else {
       NvtxRange r_agents("forward agents");
       API_TRY(agent_ffts(p, d, y, pupil, window, mu, r, al, ws, it == 0 && !spectrum_ready, st));
-      if (mu_out) API_CUDA(launch_mean(at<double>(ws, al.mures), p->looks, mu_out + it, st), "mu residual");
     }
     if (events) API_CUDA(cudaEventRecord((cudaEvent_t)events[4 * it + 1], st), "event");
     if (ss) {
@@ -855,10 +854,13 @@ static clamp_status iterate_impl(const clamp_params* p, const Derived& d, int k_
     }
     NvtxRange r_mace("prox + MACE step");
     PassC c = passc_args(p, d, al, ws, mu, r, w, wbar, k);
+    if (ce_out || (mu_out && !noap)) {
+      c.ticket = at<unsigned>(ws, al.err) + 1;
+      c.ce_out = ce_out ? ce_out + it : nullptr;
+      c.mures = at<double>(ws, al.mures);
+      c.mu_out = mu_out && !noap ? mu_out + it : nullptr;
+    }
     API_CUDA(launch_pass_c_fused(d.g, c, st), "fused prox + MACE pass");
-    if (ce_out)
-      API_CUDA(launch_ce_final(c.part_num, c.part_den, passc_fused_blocks(n, p->looks), ce_out + it, st),
-               "CE residual");
     if (events) API_CUDA(cudaEventRecord((cudaEvent_t)events[4 * it + 3], st), "event");
   }
   return CLAMP_OK;
@@ -875,7 +877,7 @@ clamp_status recon_enqueue(const clamp_params* p, const ReconPlan& d, const floa
   float* r = at<float>(ws, rl.r);
   float* w = at<float>(ws, rl.w);
   const long long n = (long long)p->nx * p->ny * p->nz;
-  API_CUDA(cudaMemsetAsync(at<int>(aws, al.err), 0, sizeof(int), st), "memset");
+  API_CUDA(cudaMemsetAsync(at<int>(aws, al.err), 0, 2 * sizeof(int), st), "memset");   // error word, residual ticket
   API_TRY(do_init_warm(p, d, y, pupil, window, r_init, mu, r, w, al, aws, st));
   if (p->max_iters == 0)
     API_CUDA(cudaMemcpyAsync(r_out, r + (long long)p->looks * n, n * sizeof(float), cudaMemcpyDeviceToDevice, st),
@@ -908,7 +910,7 @@ extern "C" clamp_status clamp_iterate(const clamp_params* p, int32_t k_first, in
   cudaStream_t st = (cudaStream_t)stream;
   Derived d;
   API_TRY(recon_prepare(p, pupil, window, st, &d));
-  API_CUDA(cudaMemsetAsync(at<int>(ws, agent_layout(p).err), 0, sizeof(int), st), "memset");
+  API_CUDA(cudaMemsetAsync(at<int>(ws, agent_layout(p).err), 0, 2 * sizeof(int), st), "memset");   // error word, residual ticket
   return iterate_impl(p, d, k_first, iters, y, pupil, window, den, reinterpret_cast<float2*>(mu), r, w, wbar, ce_out,
                       mu_out, ws, events, false, st);
 }
@@ -931,7 +933,7 @@ static clamp_status reconstruct_impl(const clamp_params* p, const float* y, cons
   Derived d;
   if (plan) d = *plan;
   else API_TRY(recon_prepare(p, pupil, window, st, &d));
-  API_CUDA(cudaMemsetAsync(at<int>(aws, al.err), 0, sizeof(int), st), "memset");
+  API_CUDA(cudaMemsetAsync(at<int>(aws, al.err), 0, 2 * sizeof(int), st), "memset");   // error word, residual ticket
   API_TRY(do_init_warm(p, d, y, pupil, window, r_init, mu, r, w, al, aws, st));
   if (p->max_iters == 0) {
     // r* = wbar of the initial state = r0

@@ -803,6 +803,50 @@ int passc_fused_blocks(long long n, int L) {
   return (int)(b < cap ? b : cap);
 }
 
+// End of a fused pass: the last CTA adds up the CTAs' convergence-error partials (in a fixed
+// order) and the looks' mu-residuals, which took two launches more per iteration (11 us of 56 on a
+// small scene).  Call after block_reduce_store.
+__device__ __forceinline__ void pass_c_residuals(const PassC& c, int L) {
+  if (!c.ticket) return;
+  __shared__ bool s_last;
+  __shared__ double red[NT / 32][2];
+  __threadfence();   // the partial sums, by the threads that wrote them
+  __syncthreads();
+  if (threadIdx.x == 0) s_last = atomicInc(c.ticket, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double a = 0, b = 0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += NT) {
+    a += __ldcg(&c.part_num[i]);
+    b += __ldcg(&c.part_den[i]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    red[warp][0] = a;
+    red[warp][1] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && c.ce_out) {
+    double num = 0, den = 0;
+    for (int w = 0; w < NT / 32; ++w) {
+      num += red[w][0];
+      den += red[w][1];
+    }
+    *c.ce_out = den > 0 ? sqrt(num / den) : 0.0;
+  }
+  if (threadIdx.x == 32 && c.mu_out) {
+    double m = 0;
+    for (int l = 0; l < L; ++l) m += c.mures[l];
+    *c.mu_out = m / L;
+  }
+}
+
 // Each thread walks the L looks of one voxel at a time.  The look loops are software-
 // pipelined: look l + 1's loads are issued before look l's arithmetic and stores (the
 // arrays do not alias), so two looks' loads are in flight per thread.
@@ -902,6 +946,7 @@ __global__ void __launch_bounds__(NT) k_pass_c(Geom g, PassC c) {
   if constexpr (MACE) {
     double* const outs[2] = {c.part_num, c.part_den};
     block_reduce_store<2>(acc, outs, blockIdx.x);
+    if constexpr (PROX) pass_c_residuals(c, L);
   }
 }
 
@@ -1047,6 +1092,7 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
   if constexpr (MACE) {
     double* const outs[2] = {c.part_num, c.part_den};
     block_reduce_store<2>(acc, outs, blockIdx.x);
+    if constexpr (PROX) pass_c_residuals(c, L);
   }
 }
 

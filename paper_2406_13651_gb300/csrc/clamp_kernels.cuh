@@ -127,6 +127,9 @@ struct BandArgs {
   float inv_nv, floor, sc_x, sc_y, sc_z;
   double *s1, *s2, *s3, *s4;  // partials: s1, s3 [L][px]; s2, s4 [L][pS]
   int px;
+  float nv;                   // sigma_w^2
+  float* gamma;               // [L] step out
+  double* mures;              // [L] mu-residual out (counts the look's finished CTAs until then)
 };
 BandShape band_shape(const float* pupil_host, int nx, int ny);
 size_t band_table_bytes(const BandShape& b, int nx, int ny);
@@ -183,6 +186,11 @@ struct PassC {
   int* err;          // device error word (non-finite)
   int exact_prox;    // 1: exact cubic-root prox instead of the quadratic-surrogate step
   int closed_mu;     // 1: mu = d / (1 + sigma_w^2 / (r' + sigma_w^2)) with d holding F^H y (no aperture)
+  // Fused pass: the last CTA to finish adds up the iteration's residuals (null: not asked for).
+  unsigned* ticket;      // zero before the pass; left at zero
+  double* ce_out;        // convergence error
+  const double* mures;   // [L] mu-residuals and their mean
+  double* mu_out;
 };
 int passc_blocks(long long n);
 // CTAs (and CE partial sums) of launch_pass_c_fused; at most passc_blocks(n).
