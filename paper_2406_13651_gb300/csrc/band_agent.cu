@@ -514,18 +514,40 @@ cudaError_t run_x(const BandArgs& a, int L, int mode, int variant, cudaStream_t 
 
 }  // namespace
 
-BandShape band_shape(const float* pupil_host, int nx, int ny) {
+// One pass along the rows, eight columns at a time (independent sums, so the loop vectorises): the GPU
+// waits meanwhile.  A chain of additions and a second, column-wise walk took about 100 us at
+// 192x192, an eighth of a caller's iteration there.
+BandShape band_shape(const float* pupil_host, int nx, int ny, double* sum_sq) {
   BandShape b{};
-  int nS = 0, nbx = 0;
-  for (int kx = 0; kx < nx; ++kx) {
-    bool any = false;
-    for (int ky = 0; ky < ny; ++ky) {
-      const bool nz = pupil_host[ky * nx + kx] != 0.0f;
-      any |= nz;
-      nS += nz;
+  constexpr int K = 8;
+  std::vector<int> any(nx, 0);
+  double s[K] = {};
+  int cnt[K] = {};
+  for (int ky = 0; ky < ny; ++ky) {
+    const float* row = pupil_host + (size_t)ky * nx;
+    int kx = 0;
+    for (; kx + K <= nx; kx += K)
+      for (int j = 0; j < K; ++j) {
+        const float v = row[kx + j];
+        const int set = v != 0.0f;
+        s[j] += (double)v * v;
+        cnt[j] += set;
+        any[kx + j] |= set;
+      }
+    for (; kx < nx; ++kx) {
+      s[0] += (double)row[kx] * row[kx];
+      cnt[0] += row[kx] != 0.0f;
+      any[kx] |= row[kx] != 0.0f;
     }
-    nbx += any;
   }
+  int nS = 0, nbx = 0;
+  double sum = 0;
+  for (int j = 0; j < K; ++j) {
+    nS += cnt[j];
+    sum += s[j];
+  }
+  for (int kx = 0; kx < nx; ++kx) nbx += any[kx];
+  *sum_sq = sum;
   b.nS = nS;
   b.nSp = (nS + BC - 1) / BC * BC;
   b.nbx = nbx;

@@ -264,10 +264,8 @@ clamp_status recon_prepare_host(const clamp_params* p, const float* hp, const fl
   d->band_fits = false;
   const size_t np = (size_t)p->nx * p->ny;
   double sp = 0, sw = 0;
-  for (size_t i = 0; i < np; ++i) {
-    if (!isfinite(hp[i])) return api_fail(CLAMP_EINVAL, "pupil has a non-finite value");
-    sp += (double)hp[i] * hp[i];
-  }
+  d->band = band_shape(hp, p->nx, p->ny, &sp);
+  if (!isfinite(sp)) return api_fail(CLAMP_EINVAL, "pupil has a non-finite value");   // squares of floats do not overflow
   for (int i = 0; i < p->nz; ++i) {
     if (!isfinite(hw[i])) return api_fail(CLAMP_EINVAL, "window has a non-finite value");
     sw += (double)hw[i] * hw[i];
@@ -275,7 +273,6 @@ clamp_status recon_prepare_host(const clamp_params* p, const float* hp, const fl
   const double alpha = (sp / np) * (sw / p->nz);
   if (!(alpha > 0)) return api_fail(CLAMP_EINVAL, "aperture is identically zero (alpha = 0)");
   d->alpha = alpha;
-  d->band = band_shape(hp, p->nx, p->ny);
   d->band_fits = band_fits(p, d->band);
   d->s.nv = p->noise_var;
   d->s.alpha = (float)alpha;

@@ -131,7 +131,8 @@ struct BandArgs {
   float* gamma;               // [L] step out
   double* mures;              // [L] mu-residual out (counts the look's finished CTAs until then)
 };
-BandShape band_shape(const float* pupil_host, int nx, int ny);
+// The support's and band's counts; *sum_sq = sum of squares, finite iff every pupil value is.
+BandShape band_shape(const float* pupil_host, int nx, int ny, double* sum_sq);
 size_t band_table_bytes(const BandShape& b, int nx, int ny);
 BandTables band_tables_at(const BandShape& b, int nx, int ny, void* base);
 int band_pS(const BandShape& b);
