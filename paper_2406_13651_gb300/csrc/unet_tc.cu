@@ -18,17 +18,21 @@
 // A CTA owns XW x 16 voxels of up to ZT planes (their accumulators fill 256 TMEM columns, so
 // two CTAs share an SM) and, for every 16-channel chunk, marches along z: each plane is
 // loaded and rounded once per chunk into a ring of four, and completes the three planes one
-// output plane needs.  While a plane's MMAs run (one thread issues them, 27 per patch, and
-// commits them to an mbarrier), the next plane's loads are in flight in registers; it is
-// stored once the MMAs of the plane before have completed.  CTAs are persistent: TMEM and
-// barriers are set up once, and the next tile's first plane is loaded under the current
-// tile's last MMAs.  Waits are bounded and set an error bit instead of hanging.
+// output plane needs.  Seven warps stage: the next plane's loads are in flight in registers
+// while a plane's MMAs run, and it is stored once the MMAs of the plane before have completed.
+// The eighth warp issues the MMAs (27 per patch, committed to an mbarrier) meanwhile: issued by
+// one of the staging threads they held up its warp, and with it all eight at the next barrier,
+// for most of the time.  CTAs are persistent: TMEM and barriers are set up once, and the next
+// tile's first plane is loaded under the current tile's last MMAs.  Waits are bounded and set an
+// error bit instead of hanging.
 //
 // For one output the MMAs accumulate chunk by chunk in tap order, as the earlier kernel's did
 // (three shifted halo copies staged per output plane, no overlap), so results are
 // the same bit for bit.  Bound: a 4 KB A operand read per MMA (32 clocks for N = 16; 0.20 ms
-// per 16 -> 16 conv at 256x256x128) and the FP32 planes' traffic (0.16 ms); measured 2.27 -> 0.55
-// ms there, 32 -> 16 2.3 -> 0.99 ms, 32 -> 32 at half size 0.42 -> 0.21 ms.
+// per 16 -> 16 conv at 256x256x128) and the FP32 planes' traffic (0.16 ms); measured there, mean of
+// two 16 -> 16 and one 32 -> 16: 0.69 ms with the MMAs issued by a staging thread, now 0.56 (32 -> 32 at
+// half size 0.23 -> 0.20).  What is left is the latency of a plane's round (load, store, barrier,
+// MMAs) at two CTAs per SM, which registers and shared memory allow.
 #include "../../include/clamp.h"
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
@@ -42,6 +46,7 @@ namespace clamp {
 namespace unet_tc {
 
 constexpr int UNT = 256;   // threads per CTA
+constexpr int UST = 224;   // of these stage; the last warp issues the MMAs
 constexpr uint32_t kWaitLimit = 1u << 22;
 constexpr int TROWS = 16;  // rows of a tile
 
@@ -53,7 +58,7 @@ struct UtCfg {
   static constexpr int PLANE_VEC = 2 * CG_VEC;
   static constexpr int ZT = 256 / (TX * COUT);                    // output planes whose accumulators fit 256 columns
   static constexpr int W_VEC = 27 * 2 * COUT;                     // a chunk's weights [tap][group][C_out]
-  static constexpr int TASKS = (PLANE_VEC + UNT - 1) / UNT;       // staging tasks (8 channels of a voxel) per thread
+  static constexpr int TASKS = (PLANE_VEC + UST - 1) / UST;       // staging tasks (8 channels of a voxel) per thread
   static constexpr size_t SMEM = 1024 + 16 * (size_t)(4 * PLANE_VEC + W_VEC) + 64;
   static_assert(ZT >= 1 && TX * COUT * ZT == 256, "TMEM");
   static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two CTAs per SM");
@@ -140,7 +145,7 @@ __global__ void __launch_bounds__(UNT, 2)
     const float* src = in + (long long)t.b * in_bs + (long long)(16 * c) * n + (zin ? gz * plane : 0LL);
 #pragma unroll
     for (int k = 0; k < Cfg::TASKS; ++k) {
-      const int e = tid + k * UNT;
+      const int e = tid + k * UST;
       const int cg = e / Cfg::CG_VEC, r = e % Cfg::CG_VEC;
       const int gx = t.x0 + r % P - 1, gy = t.y0 + r / P - 1;
       const bool ok = e < Cfg::PLANE_VEC && zin && gx >= 0 && gx < nx && gy >= 0 && gy < ny;
@@ -152,7 +157,7 @@ __global__ void __launch_bounds__(UNT, 2)
   auto store = [&](uint32_t slot) {
 #pragma unroll
     for (int k = 0; k < Cfg::TASKS; ++k) {
-      const int e = tid + k * UNT;
+      const int e = tid + k * UST;
       if (e < Cfg::PLANE_VEC)
         s_a[slot * Cfg::PLANE_VEC + e] = make_uint4(bf16x2(v[k][0], v[k][1]), bf16x2(v[k][2], v[k][3]),
                                                     bf16x2(v[k][4], v[k][5]), bf16x2(v[k][6], v[k][7]));
@@ -160,7 +165,7 @@ __global__ void __launch_bounds__(UNT, 2)
   };
   auto weights = [&](int c) {
     const uint4* src = wpk + (long long)c * Cfg::W_VEC;
-    for (int e = tid; e < Cfg::W_VEC; e += UNT) cp_async16(&s_w[e], &src[e]);
+    for (int e = tid; e < Cfg::W_VEC; e += UST) cp_async16(&s_w[e], &src[e]);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   // MMAs of output plane o of the tile: planes in ring slots g - 2, g - 1, g
@@ -209,7 +214,7 @@ __global__ void __launch_bounds__(UNT, 2)
   uint32_t issued = 0;    // commits issued; commit k is on mbar[k & 1], phase k >> 1
   uint32_t waited = 0;    // commits waited for
   bool aborted = false;
-  // bounded wait (thread 0) for every commit but the newest `keep`, then a barrier
+  // bounded wait (thread 0) for every commit but the newest `keep`
   auto drain = [&](uint32_t keep) {
     if (tid == 0)
       for (uint32_t k = waited; k + keep < issued; ++k)
@@ -218,15 +223,15 @@ __global__ void __launch_bounds__(UNT, 2)
           break;
         }
     if (issued > keep && issued - keep > waited) waited = issued - keep;
-    __syncthreads();
-    tc::fence_after_sync();
-    return *abort_flag == 0;
   };
+  const bool stager = tid < UST;
   int tile = blockIdx.x;   // < ntiles: the grid has at most a CTA per tile
   bool pending = false;    // the previous tile's epilogue is not done (its MMAs may be in flight)
-  load(at(tile), 0, 0);
-  weights(0);
-  store(0);
+  if (stager) {
+    load(at(tile), 0, 0);
+    weights(0);
+    store(0);
+  }
   tc::fence_proxy_async();
   __syncthreads();
   while (tile < ntiles && !aborted) {
@@ -237,39 +242,55 @@ __global__ void __launch_bounds__(UNT, 2)
       // the next arrival's loads
       const bool last = i + 1 == nchunks * per_chunk;
       const bool more = !last || next < ntiles;
-      if (!last) load(cur, (i + 1) / per_chunk, (i + 1) % per_chunk);
-      else if (more) load(at(next), 0, 0);
-      bool did = false;
-      if (p >= 2 && cur.z0 + p - 2 < nz) {
-        did = true;
-        if (tid == 0) {
-          tc::fence_after_sync();
-          issue(g, c, p - 2);
-          tc::mma_commit(&mbar[issued & 1u]);
-        }
+      if (stager) {
+        if (!last) load(cur, (i + 1) / per_chunk, (i + 1) % per_chunk);
+        else if (more) load(at(next), 0, 0);
+      }
+      const bool did = p >= 2 && cur.z0 + p - 2 < nz;
+      if (did) {
         ++issued;
+        if (!stager) {
+          if (tc::elect_one()) {
+            tc::fence_after_sync();
+            issue(g, c, p - 2);
+            tc::mma_commit(&mbar[(issued - 1) & 1u]);
+          }
+          __syncwarp();
+        }
       }
       // the slot of arrival g + 1 held arrival g - 3, last read by the MMAs of arrival g - 1
-      if (!drain(did ? 1u : 0u)) {
-        aborted = true;
-        break;
+      drain(did ? 1u : 0u);
+      if (did) {
+        if (stager) asm volatile("bar.sync 1, %0;" ::"n"(UST) : "memory");
+      } else {
+        __syncthreads();
       }
-      if (p == 0 && nchunks > 1 && (c > 0 || pending)) weights(c);   // the previous chunk's MMAs are done
-      if (p == 0 && pending) {
-        epilogue(at(tile - (int)gridDim.x));
-        pending = false;
+      tc::fence_after_sync();
+      if ((did && !stager) || *abort_flag == 0) {   // a wait that gave up: nothing more is written, all leave below
+        if (p == 0 && nchunks > 1 && (c > 0 || pending) && stager) weights(c);   // the previous chunk's MMAs are done
+        if (p == 0 && pending) {
+          epilogue(at(tile - (int)gridDim.x));
+          pending = false;
+        }
+        if (more && stager) store((g + 1) & 3u);
+        if (p <= 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
       }
-      if (more) store((g + 1) & 3u);
-      if (p <= 1) asm volatile("cp.async.wait_group 0;" ::: "memory");
       tc::fence_proxy_async();
       tc::fence_before_sync();
       __syncthreads();
+      if (*abort_flag != 0) {
+        aborted = true;
+        break;
+      }
     }
     pending = true;
     tile = next;
   }
   if (!aborted && pending) {
-    if (drain(0)) epilogue(at(tile - (int)gridDim.x));
+    drain(0);
+    __syncthreads();
+    tc::fence_after_sync();
+    if (*abort_flag == 0) epilogue(at(tile - (int)gridDim.x));
     else aborted = true;
   }
   if (aborted && tid == 0) {
