@@ -27,6 +27,23 @@ __device__ __forceinline__ float opr(float x, int bf) {
   return bf ? __bfloat162float(__float2bfloat16_rn(x)) : x;
 }
 
+// Two packed FP32 values; fma2 rounds each half as fmaf does.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 enum LayerKind { CONV3 = 0, TCONV = 1, CONV1 = 2 };
 struct Layer {
   int kind, ci, co;
@@ -411,81 +428,132 @@ __global__ void __launch_bounds__(UT) k_pool_bwd(const float* __restrict__ dout,
 
 // Transposed conv, kernel 2^3, stride 2: out[b][co][2v + d] = bias[co] + sum_ci W[ci][co][d] in[b][ci][v].
 // (nx, ny, nz) are the OUTPUT dimensions.  A CTA keeps the weights of 16 output channels in shared
-// memory and walks runs of 64 input voxels (staged once for all outputs); a thread makes the
-// 8 children of one voxel for 4 output channels, so an input value feeds 32 FMAs where a
-// thread per output read it, its weight and both their addresses for one.  The two at
-// 256x256x128: 5.33 -> 0.64 ms.
-constexpr int TF_V = 64, TF_CO = 16;
-static size_t tconv_fwd_smem(int ci) { return sizeof(float) * (size_t)ci * (TF_CO * 8 + TF_V); }
-__global__ void __launch_bounds__(UT) k_tconv_fwd(const float* __restrict__ in, int ci_n, float* __restrict__ out, long long out_bs,
-                                                  int co_n, const float* __restrict__ W, const float* __restrict__ bias, int B, int nx,
-                                                  int ny, int nz, int bf) {
+// memory and walks runs of 64 VPT input voxels; a thread makes the 8 children of VPT voxels for
+// 4 output channels, two children to an FFMA2 (fma.rn.f32x2: each half rounded as fmaf rounds), so
+// eight 16-byte weight loads feed 32 VPT multiply-adds.  The next run's inputs are on their
+// way (cp.async, two buffers where they fit) while this one's are used.  Bound by the
+// multiply-adds and the output's stores: 32 -> 16 at 256x256x128 115 us of FMAs, 99 us of HBM; 434 us
+// with one voxel per thread, scalar FMAs and nothing in flight, now 321 (64 -> 32 at half size 213 ->
+// 158); the stores of a run wait for its last multiply-add.
+constexpr int TF_CO = 16;
+static size_t tconv_fwd_smem(int ci, int vpt, int nbuf) { return sizeof(float) * (size_t)ci * (TF_CO * 8 + nbuf * 64 * vpt); }
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+template <int VPT>
+__global__ void __launch_bounds__(UT, 2) k_tconv_fwd(const float* __restrict__ in, int ci_n, float* __restrict__ out, long long out_bs,
+                                                     int co_n, const float* __restrict__ W, const float* __restrict__ bias, int B,
+                                                     int nx, int ny, int nz, int bf, int nbuf, int vec) {
+  constexpr int V = 64 * VPT;
   extern __shared__ __align__(16) float tf_sm[];
   float* s_w = tf_sm;                       // [ci][TF_CO][8]
-  float* s_x = tf_sm + ci_n * TF_CO * 8;    // [ci][TF_V]
+  float* s_x = tf_sm + ci_n * TF_CO * 8;    // [nbuf][ci][V]
   const int ix = nx / 2, iy = ny / 2, iz = nz / 2, in_n = ix * iy * iz;
   const long long plane = (long long)nx * ny, n = plane * nz;
-  const int co0 = blockIdx.y * TF_CO, runs = (in_n + TF_V - 1) / TF_V;
+  const int co0 = blockIdx.y * TF_CO, per_b = (in_n + V - 1) / V;
+  const long long runs = (long long)B * per_b;
   for (int e = threadIdx.x; e < ci_n * TF_CO * 8; e += UT) {
     const int d = e % 8, co = (e / 8) % TF_CO, ci = e / (8 * TF_CO);
     s_w[e] = co0 + co < co_n ? opr(__ldg(&W[((long long)ci * co_n + co0 + co) * 8 + d]), bf) : 0.f;
   }
-  const int vi = threadIdx.x % TF_V, cog = threadIdx.x / TF_V;   // this thread's voxel of the run, its 4 channels
+  auto stage = [&](long long r, float* to) {   // voxels past the sample's end are left as they are: not used
+    const int b = (int)(r / per_b), v0 = (int)(r % per_b) * V;
+    const float* src = in + (long long)b * ci_n * in_n + v0;
+    if (vec) {   // in_n a multiple of four, 16-byte aligned
+      for (int e = threadIdx.x; e < ci_n * (V / 4); e += UT) {
+        const int c = e / (V / 4), q = 4 * (e % (V / 4));
+        if (v0 + q < in_n) cp_async16(to + c * V + q, src + (long long)c * in_n + q);
+      }
+    } else {
+      for (int e = threadIdx.x; e < ci_n * V; e += UT)
+        if (v0 + e % V < in_n) cp_async4(to + e, src + (long long)(e / V) * in_n + e % V);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const int vi = threadIdx.x % 64, cog = threadIdx.x / 64;   // this thread's voxels vi + 64 k of the run, its 4 channels
   float bv[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) bv[j] = co0 + 4 * cog + j < co_n ? __ldg(&bias[co0 + 4 * cog + j]) : 0.f;
-  for (long long r = blockIdx.x; r < (long long)B * runs; r += gridDim.x) {
-    const int b = (int)(r / runs), v0 = (int)(r % runs) * TF_V;
+  int cur = 0;
+  if (blockIdx.x < runs) stage(blockIdx.x, s_x);
+  for (long long r = blockIdx.x; r < runs; r += gridDim.x) {
+    const bool more = r + gridDim.x < runs;
+    if (nbuf == 2 && more) {
+      stage(r + gridDim.x, s_x + (cur ^ 1) * ci_n * V);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
     __syncthreads();
-    const float* src = in + (long long)b * ci_n * in_n + v0;
-    for (int e = threadIdx.x; e < ci_n * TF_V; e += UT)
-      s_x[e] = v0 + e % TF_V < in_n ? opr(__ldg(&src[(long long)(e / TF_V) * in_n + e % TF_V]), bf) : 0.f;
-    __syncthreads();
-    const int v = v0 + vi;
-    if (v >= in_n) continue;
-    float acc[4][8];
+    unsigned long long acc[VPT][4][4];   // [voxel][channel][pair of children]
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int k = 0; k < VPT; ++k)
 #pragma unroll
-      for (int d = 0; d < 8; ++d) acc[j][d] = bv[j];
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[k][j][q] = pack2(bv[j], bv[j]);
+    const float* xs = s_x + cur * ci_n * V + vi;
 #pragma unroll 2
     for (int ci = 0; ci < ci_n; ++ci) {
-      const float x = s_x[ci * TF_V + vi];
-      const float4* w = reinterpret_cast<const float4*>(s_w + (ci * TF_CO + 4 * cog) * 8);
+      unsigned long long x[VPT];
+#pragma unroll
+      for (int k = 0; k < VPT; ++k) {
+        const float xv = opr(xs[ci * V + 64 * k], bf);
+        x[k] = pack2(xv, xv);
+      }
+      const ulonglong2* w = reinterpret_cast<const ulonglong2*>(s_w + (ci * TF_CO + 4 * cog) * 8);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float4 w0 = w[2 * j], w1 = w[2 * j + 1];
-        acc[j][0] = fmaf(w0.x, x, acc[j][0]);
-        acc[j][1] = fmaf(w0.y, x, acc[j][1]);
-        acc[j][2] = fmaf(w0.z, x, acc[j][2]);
-        acc[j][3] = fmaf(w0.w, x, acc[j][3]);
-        acc[j][4] = fmaf(w1.x, x, acc[j][4]);
-        acc[j][5] = fmaf(w1.y, x, acc[j][5]);
-        acc[j][6] = fmaf(w1.z, x, acc[j][6]);
-        acc[j][7] = fmaf(w1.w, x, acc[j][7]);
+        const ulonglong2 w0 = w[2 * j], w1 = w[2 * j + 1];
+#pragma unroll
+        for (int k = 0; k < VPT; ++k) {
+          acc[k][j][0] = fma2(w0.x, x[k], acc[k][j][0]);
+          acc[k][j][1] = fma2(w0.y, x[k], acc[k][j][1]);
+          acc[k][j][2] = fma2(w1.x, x[k], acc[k][j][2]);
+          acc[k][j][3] = fma2(w1.y, x[k], acc[k][j][3]);
+        }
       }
     }
-    const int x = v % ix, y = (v / ix) % iy, z = v / (ix * iy);
-    float* o = out + (long long)b * out_bs + (long long)(co0 + 4 * cog) * n + 2 * z * plane + (long long)(2 * y) * nx + 2 * x;
+    __syncthreads();   // this buffer's readers are done
+    if (nbuf == 2) cur ^= 1;
+    else if (more) stage(r + gridDim.x, s_x);
+    const int b = (int)(r / per_b), v0 = (int)(r % per_b) * V;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (co0 + 4 * cog + j >= co_n) continue;
+    for (int k = 0; k < VPT; ++k) {
+      const int v = v0 + vi + 64 * k;
+      if (v >= in_n) continue;
+      const int x = v % ix, y = (v / ix) % iy, z = v / (ix * iy);
+      float* o = out + (long long)b * out_bs + (long long)(co0 + 4 * cog) * n + 2 * z * plane + (long long)(2 * y) * nx + 2 * x;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        *reinterpret_cast<float2*>(o + j * n + (q >> 1) * plane + (q & 1) * nx) = make_float2(acc[j][2 * q], acc[j][2 * q + 1]);
+      for (int j = 0; j < 4; ++j) {
+        if (co0 + 4 * cog + j >= co_n) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<float2*>(o + j * n + (q >> 1) * plane + (q & 1) * nx) = unpack2(acc[k][j][q]);
+      }
     }
   }
 }
 
 static cudaError_t tconv_fwd(const float* in, int ci, float* out, long long out_bs, int co, const float* W, const float* bias,
                              int B, int nx, int ny, int nz, int bf, cudaStream_t st) {
-  const size_t smem = tconv_fwd_smem(ci);
-  cudaError_t e = cudaFuncSetAttribute(k_tconv_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // two voxels per thread in two buffers where two CTAs fit an SM, else one voxel and one buffer
+  const bool two = 2 * (tconv_fwd_smem(ci, 2, 2) + 1024) <= 227 * 1024;
+  const int vpt = two ? 2 : 1, nbuf = two ? 2 : 1;
+  auto kern = two ? k_tconv_fwd<2> : k_tconv_fwd<1>;
+  const size_t smem = tconv_fwd_smem(ci, vpt, nbuf);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const long long runs = (long long)B * (((long long)nx * ny * nz / 8 + TF_V - 1) / TF_V);
+  const long long in_n = (long long)nx * ny * nz / 8;
+  const long long runs = (long long)B * ((in_n + 64 * vpt - 1) / (64 * vpt));
   const int cb = (co + TF_CO - 1) / TF_CO;
-  const dim3 grid((unsigned)std::min(runs, std::max(1LL, 152LL * 6 / cb)), cb);
-  k_tconv_fwd<<<grid, UT, smem, st>>>(in, ci, out, out_bs, co, W, bias, B, nx, ny, nz, bf);
+  const int per_sm = two ? 2 : 6;
+  const dim3 grid((unsigned)std::min(runs, std::max(1LL, 152LL * per_sm / cb)), cb);
+  const int vec = in_n % 4 == 0 && (uintptr_t)in % 16 == 0;
+  kern<<<grid, UT, smem, st>>>(in, ci, out, out_bs, co, W, bias, B, nx, ny, nz, bf, nbuf, vec);
   return cudaGetLastError();
 }
 
