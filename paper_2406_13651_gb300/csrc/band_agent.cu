@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(1024) k_band_tables(const float* __restrict__ 
 
 template <int N>
 __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_inv(BandArgs a, const float2* __restrict__ twB) {
+  after_previous();
   [[maybe_unused]] const long long nL = (long long)a.L * a.n, sL = (long long)a.L * a.nz * a.t.nSp;   // buffer extents
   constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2;
   float2* sm = reinterpret_cast<float2*>(band_smem);
@@ -217,6 +218,7 @@ __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_inv(
 // INV: Gz on the support -> E on the band (zero off the support).  !INV: band -> support.
 template <int N, bool INV>
 __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_y(BandArgs a, const float2* __restrict__ twB) {
+  after_previous();
   [[maybe_unused]] const long long sL = (long long)a.L * a.nz * a.t.nSp,
                                    bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
   constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2;
@@ -279,6 +281,7 @@ template <int N, int V> struct RowCta {
 template <int N, int MODE, int V>
 __global__ void __launch_bounds__(RowCta<N, V>::THREADS, RowCta<N, V>::MINB)
     k_band_x(BandArgs a, const float2* __restrict__ twA, const float2* __restrict__ twB) {
+  after_previous();
   [[maybe_unused]] const long long nL = (long long)a.L * a.n, bL = (long long)a.L * a.nz * a.ny * a.t.nbxp;   // buffer extents
   constexpr int R1 = RRow<N>::R1, R2 = RRow<N>::R2, T = RRow<N>::T, LINES = RowCta<N, V>::LINES;
   constexpr bool LATE = V == 2 && MODE == BAND_GRAD;   // mu, r' read after the inverse transform
@@ -403,6 +406,7 @@ __device__ __forceinline__ void look_step(const BandArgs& a, int l, int pS) {
 // BAND_GRAD: F d on the support (in place), S2 = ||a F d||^2 and the look's step.  BAND_SPEC: writes M.
 template <int N, int MODE>
 __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_fwd(BandArgs a, const float2* __restrict__ twB) {
+  after_previous();
   [[maybe_unused]] const long long sL = (long long)a.L * a.nz * a.t.nSp;   // buffer extent
   constexpr int R1 = RCol<N>::R1, R2 = RCol<N>::R2;
   float2* sm = reinterpret_cast<float2*>(band_smem);
@@ -471,10 +475,9 @@ cudaError_t run_z(const BandArgs& a, int L, bool inverse, int mode, cudaStream_t
     constexpr int N = decltype(NC)::value, TH = RCol<N>::THREADS;
     constexpr size_t smem = RCol<N>::SMEM;   // at most 33 KB: within the default limit
     const dim3 grid(a.t.nSp / BC, L);
-    if (inverse) k_band_z_inv<N><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
-    else if (mode == BAND_GRAD) k_band_z_fwd<N, BAND_GRAD><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
-    else k_band_z_fwd<N, BAND_SPEC><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
-    return cudaGetLastError();
+    if (inverse) return launch_after(k_band_z_inv<N>, grid, TH, smem, st, a, twiddle_table_b(N));
+    if (mode == BAND_GRAD) return launch_after(k_band_z_fwd<N, BAND_GRAD>, grid, TH, smem, st, a, twiddle_table_b(N));
+    return launch_after(k_band_z_fwd<N, BAND_SPEC>, grid, TH, smem, st, a, twiddle_table_b(N));
   });
 }
 
@@ -483,9 +486,8 @@ cudaError_t run_y(const BandArgs& a, int L, bool inverse, cudaStream_t st) {
     constexpr int N = decltype(NC)::value, TH = RCol<N>::THREADS;
     constexpr size_t smem = RCol<N>::SMEM;
     const dim3 grid(a.t.nbxp / BC, a.nz, L);
-    if (inverse) k_band_y<N, true><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
-    else k_band_y<N, false><<<grid, TH, smem, st>>>(a, twiddle_table_b(N));
-    return cudaGetLastError();
+    if (inverse) return launch_after(k_band_y<N, true>, grid, TH, smem, st, a, twiddle_table_b(N));
+    return launch_after(k_band_y<N, false>, grid, TH, smem, st, a, twiddle_table_b(N));
   });
 }
 
@@ -494,8 +496,7 @@ cudaError_t launch_x(const BandArgs& a, int L, cudaStream_t st) {
   using Cta = RowCta<N, V>;
   static_assert(Cta::SMEM <= 48 * 1024, "default shared-memory limit");
   const unsigned grid = (unsigned)((long long)L * a.nz * a.ny / Cta::LINES);
-  k_band_x<N, MODE, V><<<grid, Cta::THREADS, Cta::SMEM, st>>>(a, twiddle_table_a(N), twiddle_table_b(N));
-  return cudaGetLastError();
+  return launch_after(k_band_x<N, MODE, V>, grid, Cta::THREADS, Cta::SMEM, st, a, twiddle_table_a(N), twiddle_table_b(N));
 }
 
 cudaError_t run_x(const BandArgs& a, int L, int mode, int variant, cudaStream_t st) {

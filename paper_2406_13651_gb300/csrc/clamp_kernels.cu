@@ -962,6 +962,7 @@ constexpr int kPassCPrefetch = 6;   // looks ahead that the look loop prefetches
 
 template <bool PROX, bool MACE>
 __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
+  after_previous();
   const long long n2 = g.n / 2;
   const int L = g.L;
   const float2* __restrict__ Wi = reinterpret_cast<const float2*>(c.w);
@@ -1125,7 +1126,7 @@ static bool pass_c_pairs(const Geom& g, const PassC& c, bool prox, bool mace) {
 cudaError_t launch_pass_c_fused(const Geom& g, const PassC& c, cudaStream_t st) {
   const int nb = passc_fused_blocks(g.n, g.L);
   if (c.exact_prox) k_pass_c<true, true, true><<<nb, NT, 0, st>>>(g, c);
-  else if (pass_c_pairs(g, c, true, true)) k_pass_c_pair<true, true><<<nb, NT, 0, st>>>(g, c);
+  else if (pass_c_pairs(g, c, true, true)) return launch_after(k_pass_c_pair<true, true>, nb, NT, 0, st, g, c);
   else k_pass_c<true, true><<<nb, NT, 0, st>>>(g, c);
   return cudaGetLastError();
 }
