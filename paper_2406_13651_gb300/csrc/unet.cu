@@ -559,14 +559,16 @@ static cudaError_t tconv_fwd(const float* in, int ci, float* out, long long out_
 
 // din[b][ci][v] = sum_co sum_d W[ci][co][d] dout[b][co][2v + d]  ((nx, ny, nz) = output dims).  A CTA
 // keeps the weights of CI = 32 input channels in shared memory (16 above 128 output channels);
-// a thread owns one voxel and CI / 4 input channels, so a voxel's 8 children (four 8-byte
-// loads, shared by the four threads of the voxel through L1) feed 64 FMAs.  The two
-// at 24 x 64x64x32: 1.22 -> 0.38 ms.
-constexpr int TD_V = 64;
-template <int CI>
-__global__ void __launch_bounds__(UT) k_tconv_dgrad(const float* __restrict__ dout, long long dout_bs, int co_n, float* __restrict__ din,
-                                                    int ci_n, const float* __restrict__ W, int B, int nx, int ny, int nz, int bf) {
-  constexpr int PER = CI / 4;
+// a thread owns TD_K voxels and CI / 4 input channels, so a weight loaded serves TD_K FMAs (shared
+// memory returns one float per lane and clock to the SM's four schedulers together) and a
+// voxel's 8 children (four 8-byte loads, shared by the voxel's four threads through L1)
+// CI / 4 each.  The two at 24 x 64x64x32 (65 us of FMAs): 1.22 ms, 0.38 with one voxel per
+// thread (still the better where four leave an SM without two CTAs: 64 -> 32 at 24 x 16^3 41
+// against 48 us), now 0.23.
+template <int CI, int TD_K>
+__global__ void __launch_bounds__(UT, 2) k_tconv_dgrad(const float* __restrict__ dout, long long dout_bs, int co_n, float* __restrict__ din,
+                                                       int ci_n, const float* __restrict__ W, int B, int nx, int ny, int nz, int bf) {
+  constexpr int PER = CI / 4, TD_V = 64 * TD_K;
   extern __shared__ __align__(16) float td_sm[];   // [co][CI][8]
   const int ix = nx / 2, iy = ny / 2, iz = nz / 2, in_n = ix * iy * iz;
   const long long plane = (long long)nx * ny, n = plane * nz;
@@ -576,55 +578,73 @@ __global__ void __launch_bounds__(UT) k_tconv_dgrad(const float* __restrict__ do
     td_sm[e] = ci0 + ci < ci_n ? opr(__ldg(&W[((long long)(ci0 + ci) * co_n + co) * 8 + d]), bf) : 0.f;
   }
   __syncthreads();
-  const int vi = threadIdx.x % TD_V, cig = threadIdx.x / TD_V;
+  const int vi = threadIdx.x % 64, cig = threadIdx.x / 64;
   for (long long r = blockIdx.x; r < (long long)B * runs; r += gridDim.x) {
-    const int b = (int)(r / runs), v = (int)(r % runs) * TD_V + vi;
-    if (v >= in_n) continue;
-    const int x = v % ix, y = (v / ix) % iy, z = v / (ix * iy);
-    const float* g = dout + (long long)b * dout_bs + 2 * z * plane + (long long)(2 * y) * nx + 2 * x;
-    float acc[PER];
+    const int b = (int)(r / runs), v0 = (int)(r % runs) * TD_V + vi;
+    const float* gb = dout + (long long)b * dout_bs;
+    long long off[TD_K];   // the first child of voxel v0 + 64 k; past the sample's end: its first voxel's, dropped below
 #pragma unroll
-    for (int j = 0; j < PER; ++j) acc[j] = 0.f;
-#pragma unroll 2
+    for (int k = 0; k < TD_K; ++k) {
+      const int v = v0 + 64 * k < in_n ? v0 + 64 * k : 0;
+      const int x = v % ix, y = (v / ix) % iy, z = v / (ix * iy);
+      off[k] = 2 * z * plane + (long long)(2 * y) * nx + 2 * x;
+    }
+    float acc[TD_K][PER];
+#pragma unroll
+    for (int k = 0; k < TD_K; ++k)
+#pragma unroll
+      for (int j = 0; j < PER; ++j) acc[k][j] = 0.f;
+#pragma unroll 1
     for (int co = 0; co < co_n; ++co) {
-      float gv[8];
+      const float* g = gb + (long long)co * n;
+      float gv[TD_K][8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float2 t = __ldg(reinterpret_cast<const float2*>(g + (long long)co * n + (q >> 1) * plane + (q & 1) * nx));
-        gv[2 * q] = opr(t.x, bf);
-        gv[2 * q + 1] = opr(t.y, bf);
-      }
+      for (int k = 0; k < TD_K; ++k)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 t = __ldg(reinterpret_cast<const float2*>(g + off[k] + (q >> 1) * plane + (q & 1) * nx));
+          gv[k][2 * q] = opr(t.x, bf);
+          gv[k][2 * q + 1] = opr(t.y, bf);
+        }
       const float4* w = reinterpret_cast<const float4*>(td_sm + (co * CI + PER * cig) * 8);
 #pragma unroll
       for (int j = 0; j < PER; ++j) {
         const float4 w0 = w[2 * j], w1 = w[2 * j + 1];
-        acc[j] = fmaf(w0.x, gv[0], acc[j]);
-        acc[j] = fmaf(w0.y, gv[1], acc[j]);
-        acc[j] = fmaf(w0.z, gv[2], acc[j]);
-        acc[j] = fmaf(w0.w, gv[3], acc[j]);
-        acc[j] = fmaf(w1.x, gv[4], acc[j]);
-        acc[j] = fmaf(w1.y, gv[5], acc[j]);
-        acc[j] = fmaf(w1.z, gv[6], acc[j]);
-        acc[j] = fmaf(w1.w, gv[7], acc[j]);
+#pragma unroll
+        for (int k = 0; k < TD_K; ++k) {
+          float s = acc[k][j];
+          s = fmaf(w0.x, gv[k][0], s);
+          s = fmaf(w0.y, gv[k][1], s);
+          s = fmaf(w0.z, gv[k][2], s);
+          s = fmaf(w0.w, gv[k][3], s);
+          s = fmaf(w1.x, gv[k][4], s);
+          s = fmaf(w1.y, gv[k][5], s);
+          s = fmaf(w1.z, gv[k][6], s);
+          acc[k][j] = fmaf(w1.w, gv[k][7], s);
+        }
       }
     }
-    float* o = din + ((long long)b * ci_n + ci0 + PER * cig) * in_n + v;
 #pragma unroll
-    for (int j = 0; j < PER; ++j)
-      if (ci0 + PER * cig + j < ci_n) o[(long long)j * in_n] = acc[j];
+    for (int k = 0; k < TD_K; ++k) {
+      if (v0 + 64 * k >= in_n) continue;
+      float* o = din + ((long long)b * ci_n + ci0 + PER * cig) * in_n + v0 + 64 * k;
+#pragma unroll
+      for (int j = 0; j < PER; ++j)
+        if (ci0 + PER * cig + j < ci_n) o[(long long)j * in_n] = acc[k][j];
+    }
   }
 }
 
 static cudaError_t tconv_dgrad(const float* dout, long long dout_bs, int co, float* din, int ci, const float* W, int B, int nx,
                                int ny, int nz, int bf, cudaStream_t st) {
-  const int cic = co <= 128 ? 32 : 16;
-  auto kern = cic == 32 ? k_tconv_dgrad<32> : k_tconv_dgrad<16>;
+  const int cic = co <= 128 ? 32 : 16, cb = (ci + cic - 1) / cic;
+  auto runs = [&](int k) { return (long long)B * (((long long)nx * ny * nz / 8 + 64 * k - 1) / (64 * k)); };
+  const bool four = runs(4) * cb >= 2 * 152;   // four voxels per thread
+  auto kern = cic == 32 ? (four ? k_tconv_dgrad<32, 4> : k_tconv_dgrad<32, 1>) : (four ? k_tconv_dgrad<16, 4> : k_tconv_dgrad<16, 1>);
   const size_t smem = sizeof(float) * (size_t)co * cic * 8;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  const long long runs = (long long)B * (((long long)nx * ny * nz / 8 + TD_V - 1) / TD_V);
-  const int cb = (ci + cic - 1) / cic;
-  const dim3 grid((unsigned)std::min(runs, std::max(1LL, 152LL * 6 / cb)), cb);
+  const dim3 grid((unsigned)std::min(runs(four ? 4 : 1), std::max(1LL, 152LL * 6 / cb)), cb);
   kern<<<grid, UT, smem, st>>>(dout, dout_bs, co, din, ci, W, B, nx, ny, nz, bf);
   return cudaGetLastError();
 }
@@ -1168,8 +1188,8 @@ extern "C" clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float*
 // terms further off than the tensor cores' short chains do, and a training run is meant to
 // keep following earlier ones.  The two differ by the square of the chain's length: at the
 // full-size level, whose activations carry the image's background, by up to 1.4e-5 of the
-// whole gradient at 41 k voxels a chain, at the coarser levels by 1.3e-6 at 79 k.  The
-// limits keep that at about 5e-6.
+// whole gradient at 41 k voxels a chain, at the coarser levels at 79 k by 2e-6 (median of thirteen
+// inputs at 24 x 64x64x32; at most 9.4e-6).  The limits keep it well below 2e-5.
 constexpr long long kTcChainFull = 24LL << 10, kTcChainCoarse = 160LL << 10;
 static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long in_bs, const float* g, long long g_bs,
                               float* din, long long din_bs, int B, int nx, int ny, int nz, cudaStream_t st) {
