@@ -578,7 +578,8 @@ __global__ void __launch_bounds__(TC_NT, TcPlaneCfg<CIN, NPAD>::CTAS)
   uint32_t fail_parity = 0;
 
   // a step's halo plane, loaded into registers while the MMAs of the step before it run (loaded after
-  // them: 326 us per 32 -> 32 layer at 128x128x64, now 300)
+  // them: 326 us per 32 -> 32 layer at 128x128x64, so 300; with an elected issuing thread and one
+  // waiting instead of all polling, 272)
   constexpr int PER = (Cfg::HALO_VEC + TC_NT - 1) / TC_NT;
   float4 pre[PER];
   auto load = [&](int s) {
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(TC_NT, TcPlaneCfg<CIN, NPAD>::CTAS)
     cp_async_wait_all();
     tc::fence_proxy_async();
     __syncthreads();
-    if (tid == 0) {
+    if (warp == 0 && tc::elect_one()) {
       tc::fence_after_sync();
       const uint64_t a_hi = tc::make_desc(stage_s, LBO_A, 128);
       const uint64_t a_lo = a_hi + (uint64_t)Cfg::HALO_VEC;   // start address in 16-byte units
@@ -654,8 +655,9 @@ __global__ void __launch_bounds__(TC_NT, TcPlaneCfg<CIN, NPAD>::CTAS)
       tc::mma_commit(mbar);
     }
     if (s + 1 < Cfg::STEPS) load(s + 1);
-    // every thread waits for the step's MMAs: they read the buffer the next step overwrites
-    if (!tc::mbar_wait_bounded(mbar, (uint32_t)(s & 1), kWaitLimit)) atomicOr(abort_flag, 1);
+    // the step's MMAs read the buffer the next step overwrites: one thread waits for them, the others
+    // at the barrier, which takes no issue slots from the CTAs beside this one
+    if (tid == 0 && !tc::mbar_wait_bounded(mbar, (uint32_t)(s & 1), kWaitLimit)) *abort_flag = 1;
     __syncthreads();
     if (*abort_flag) {
       aborted = true;
@@ -1161,7 +1163,7 @@ __global__ void __launch_bounds__(TC_NT) k_conv_first_tc(const float* __restrict
     // two rounds of CF1_HALF tile rows: half the TMEM per CTA, so four CTAs share an SM
 #pragma unroll 1
     for (int round = 0; round < CF1_MT / CF1_HALF; ++round) {
-      if (tid == 0) {
+      if (warp == 0 && tc::elect_one()) {
         tc::fence_after_sync();
 #pragma unroll
         for (int m = 0; m < CF1_HALF; ++m) {
