@@ -716,17 +716,17 @@ def main():
         t_it, desc = oracle_sample(wl, 2, max(4, wl.nz // 16), seed=seed)
         cpu = {"value": n * L / t_it, "unit": UNIT, "cores": oracle_threads(), "kind": "oracle", "sample": desc}
 
-    # kernels per iteration: the five agent passes and the line search, the prior (one per CNN
-    # layer; in BF16 the last hidden layer also forms the last layer's tap sums, which leaves
-    # the last layer a gather, except at 16 channels or with no hidden layer, where the tap
-    # sums are a kernel of their own), the prox/Mann pass and the CE reduction (16 at
-    # 256x256x128 with the 8-layer BF16 CNN)
+    # kernels per iteration: the five agent passes (the last one forms the line search), the prior
+    # (one per CNN layer; in BF16 the last hidden layer also forms the last layer's tap sums,
+    # which leaves the last layer a gather, except at 16 channels or with no hidden layer,
+    # where the tap sums are a kernel of their own) and the prox/Mann pass (which adds up the
+    # residuals): 14 at 256x256x128 with the 8-layer BF16 CNN
     prior_k = 1
     if wl.denoiser["kind"] == "cnn":
         nlayers = len(wl.denoiser["weights"])
         unfused = wl.denoiser["channels"] < 32 or nlayers < 3
         prior_k = nlayers + (1 if wl.denoiser.get("dtype", "fp32") == "bf16" and unfused else 0)
-    launches_per_iter = 5 + 1 + prior_k + 1 + 1
+    launches_per_iter = 5 + prior_k + 1
     warm = None
     if world == 1 and not args.no_warm_start:
         del mu, r, w, ws, y
