@@ -582,7 +582,6 @@ BandTables band_tables_at(const BandShape& b, int nx, int ny, void* base) {
   return t;
 }
 
-int band_pS(const BandShape& b) { return b.nSp / BC; }
 int band_px(int nx, int ny, int nz, int x_variant) {
   return (int)((long long)nz * ny / (x_variant == 1 ? variant_rows(nx, 2) : rows_per_cta(nx)));
 }

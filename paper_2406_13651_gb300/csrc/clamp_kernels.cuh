@@ -161,7 +161,6 @@ struct BandArgs {
 BandShape band_shape(const float* pupil_host, int nx, int ny, double* sum_sq);
 size_t band_table_bytes(const BandShape& b, int nx, int ny);
 BandTables band_tables_at(const BandShape& b, int nx, int ny, void* base);
-int band_pS(const BandShape& b);
 // S1 / S3 partial sums per look of the row pass (x_variant 0, 2: rows_per_cta rows per CTA; 1: half as many).
 int band_px(int nx, int ny, int nz, int x_variant);
 // Builds the device tables from the device pupil (one CTA).
