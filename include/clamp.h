@@ -462,10 +462,11 @@ clamp_status clamp_denoiser_create_unet(clamp_unet* net, float floor_rel, clamp_
  * operands, FP32 accumulation) wherever the level's shape allows it (nx = 16 with ny a
  * multiple of 8, or nx a multiple of 32 with ny a multiple of 4), and forms the 3x3x3 convs'
  * weight gradients there too, except where the volume gives the CUDA cores' sums long
- * chains (csrc/unet.cu, conv3_bwd); on = 0 keeps all of them on the CUDA cores.  Both round
- * the same operands to bfloat16; only the order of the FP32 sums differs.  The first conv
- * (one input channel), the transposed convs and the 1x1 conv stay on the CUDA cores.  FP32
- * networks ignore the setting. */
+ * chains or very short ones (csrc/unet.cu, conv3_bwd); on = 0 keeps all of them on the CUDA
+ * cores.  Both round the same operands to bfloat16 and add in FP32; the order differs, and the
+ * tensor cores truncate where the CUDA cores round to nearest.  The first conv (one input
+ * channel), the transposed convs and the 1x1 conv stay on the CUDA cores.  FP32 networks
+ * ignore the setting. */
 clamp_status clamp_unet_set_tensor_cores(clamp_unet* u, int32_t on);
 /* Synchronous check of the network's tensor-core waits since the last check: CLAMP_ETIMEOUT
  * (and the flag cleared) if a bounded wait gave up, else CLAMP_OK. */

@@ -53,8 +53,11 @@ cudaError_t unet_conv3_tc(const float* in, long long in_bs, int ci, float* out, 
 cudaError_t unet_conv3_cc(bool bf, const float* in, long long in_bs, int ci, float* out, long long out_bs, int co,
                           const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz,
                           cudaStream_t st);
-// dW[co][ci][27] += sum over samples and voxels of G[co][v] in[ci][v + tap] with both operands
-// rounded to BF16, on the tensor cores (any channel counts and volume).  err as above.
+// dW[co][ci][27] = sum over samples and voxels of G[co][v] in[ci][v + tap] with both operands
+// rounded to BF16, on the tensor cores (any channel counts and volume), the same bits every time.
+// part: scratch, 16-byte aligned.  err as above.
 cudaError_t unet_wgrad3_tc(const float* in, long long in_bs, int ci, const float* G, long long g_bs, int co, float* dW,
-                           int B, int nx, int ny, int nz, int* err, cudaStream_t st);
+                           int B, int nx, int ny, int nz, float* part, int* err, cudaStream_t st);
+// Floats `part` needs.
+size_t unet_wgrad3_tc_part(int ci, int co, int B, int nx, int ny, int nz);
 }  // namespace clamp

@@ -47,6 +47,7 @@ __device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigne
 enum LayerKind { CONV3 = 0, TCONV = 1, CONV1 = 2 };
 struct Layer {
   int kind, ci, co;
+  int level;    // its volume is the input's divided by this along every axis
   size_t w, b;  // offsets (floats) into the parameter buffer
   size_t nw;    // weight count
 };
@@ -1035,6 +1036,7 @@ struct Acts {
   float *ge1a, *gcat1, *gp1, *ge2a, *gcat2, *gp2, *gbta, *gbtb, *gd2a, *gd2b, *gd1a, *gd1b, *gout;
   unsigned char *arg1, *arg2;
   double* part;
+  float* shares;   // partial sums of one weight gradient
   size_t bytes;
 };
 
@@ -1061,6 +1063,14 @@ Acts acts_layout(const clamp_unet* u, int B, int nx, int ny, int nz, void* base,
   a.arg1 = reinterpret_cast<unsigned char*>(take((B * c1 * n2 + 3) / 4));
   a.arg2 = reinterpret_cast<unsigned char*>(take((B * c2 * n3 + 3) / 4));
   a.part = reinterpret_cast<double*>(take(2 * 152 * 16));
+  if (with_grads) {
+    size_t m = 0;
+    if (u->bf)
+      for (const Layer& L : u->layers)
+        if (L.kind == CONV3)
+          m = std::max(m, clamp::unet_wgrad3_tc_part(L.ci, L.co, B, nx / L.level, ny / L.level, nz / L.level));
+    a.shares = take((long long)m);
+  }
   a.bytes = off;
   return a;
 }
@@ -1082,12 +1092,12 @@ extern "C" clamp_status clamp_unet_create(int32_t c1, int32_t c2, int32_t c3, in
   u->c2 = c2;
   u->c3 = c3;
   cudaGetDevice(&u->dev);
-  const int spec[13][3] = {{CONV3, 1, c1},      {CONV3, c1, c1}, {CONV3, c1, c2}, {CONV3, c2, c2}, {CONV3, c2, c3},
-                           {CONV3, c3, c3},     {TCONV, c3, c2}, {CONV3, 2 * c2, c2}, {CONV3, c2, c2},
-                           {TCONV, c2, c1},     {CONV3, 2 * c1, c1}, {CONV3, c1, c1}, {CONV1, c1, 1}};
+  const int spec[13][4] = {{CONV3, 1, c1, 1},  {CONV3, c1, c1, 1}, {CONV3, c1, c2, 2},     {CONV3, c2, c2, 2}, {CONV3, c2, c3, 4},
+                           {CONV3, c3, c3, 4}, {TCONV, c3, c2, 2}, {CONV3, 2 * c2, c2, 2}, {CONV3, c2, c2, 2},
+                           {TCONV, c2, c1, 1}, {CONV3, 2 * c1, c1, 1}, {CONV3, c1, c1, 1}, {CONV1, c1, 1, 1}};
   size_t off = 0;
   for (auto& s : spec) {
-    Layer L{s[0], s[1], s[2], 0, 0, 0};
+    Layer L{s[0], s[1], s[2], s[3], 0, 0, 0};
     L.nw = (size_t)s[1] * s[2] * (s[0] == CONV3 ? 27 : s[0] == TCONV ? 8 : 1);
     L.w = off;
     off += L.nw;
@@ -1226,16 +1236,15 @@ extern "C" clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float*
 // conv3 backward for layer li: input `in` (ci channels, sample stride in_bs), output gradient
 // `g` (co channels, stride g_bs); writes din (if non-NULL) and accumulates dW.
 //
-// BF16 networks form dW on the tensor cores (16 -> 16 at 24 x 64x64x32: 0.29 ms, 1.46 ms on the
-// CUDA cores) unless the CUDA cores' FP32 chains are long: those round a sum of same-signed
-// terms further off than the tensor cores' short chains do, and a training run is meant to
-// keep following earlier ones.  The two differ by the square of the chain's length: at the
-// full-size level, whose activations carry the image's background, by up to 1.4e-5 of the
-// whole gradient at 41 k voxels a chain, at the coarser levels at 79 k by 2e-6 (median of thirteen
-// inputs at 24 x 64x64x32; at most 9.4e-6).  The limits keep it well below 2e-5.
-constexpr long long kTcChainFull = 24LL << 10, kTcChainCoarse = 160LL << 10;
+// BF16 networks form dW on the tensor cores (16 -> 16 at 24 x 32^3: 0.11 ms, 0.47 ms on the CUDA
+// cores) between two lengths of the CUDA cores' FP32 chains:
+//   * below 128 terms a launch more would cost what the tensor cores save (17 against 10 to 17 us), and
+//     the CUDA cores' sums are as exact (64 -> 64 at chains of 85: 4.3e-8 of FP64 against 4.5e-8);
+//   * the longer chains are the less exact of the two, but they are what earlier training runs
+//     followed, and a gradient that leaves them moves by their whole error.
+constexpr long long kTcChainMin = 128, kTcChainFull = 24LL << 10, kTcChainCoarse = 160LL << 10;
 static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long in_bs, const float* g, long long g_bs,
-                              float* din, long long din_bs, int B, int nx, int ny, int nz, cudaStream_t st) {
+                              float* din, long long din_bs, int B, int nx, int ny, int nz, float* part, cudaStream_t st) {
   const Layer& L = u->layers[li];
   const bool bf = u->bf != 0;
   if (din) {
@@ -1243,9 +1252,10 @@ static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long 
     U_TRY(cudaGetLastError());
     U_TRY(conv3(bf, g, g_bs, L.co, din, din_bs, L.ci, u->flip, nullptr, false, B, nx, ny, nz, st, u->ctx()));
   }
-  const long long chain = li <= 1 || li >= 10 ? kTcChainFull : kTcChainCoarse;
-  if (u->ctx().on && (long long)B * nx * ny * nz <= chain * wgrad3_shares(L.ci, L.co, B, ny, nz))
-    U_TRY(clamp::unet_wgrad3_tc(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->err, st));
+  const long long shares = wgrad3_shares(L.ci, L.co, B, ny, nz), voxels = (long long)B * nx * ny * nz;
+  const long long most = L.level == 1 ? kTcChainFull : kTcChainCoarse;
+  if (u->ctx().on && voxels >= kTcChainMin * shares && voxels <= most * shares)
+    U_TRY(clamp::unet_wgrad3_tc(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, part, u->err, st));
   else
     U_TRY(wgrad3(in, in_bs, L.ci, g, g_bs, L.co, u->g + L.w, B, nx, ny, nz, u->bf, st));
   return CLAMP_OK;
@@ -1283,10 +1293,10 @@ extern "C" clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const
       a.d1b, c1, a.gout, W(12), a.gd1b, u->g + u->layers[12].w, dB(12), dB(11), B, n1, bf);
   U_TRY(cudaGetLastError());
   // decoder level 1
-  s = conv3_bwd(u, 11, a.d1a, c1 * n1, a.gd1b, c1 * n1, a.gd1a, c1 * n1, B, nx, ny, nz, st);
+  s = conv3_bwd(u, 11, a.d1a, c1 * n1, a.gd1b, c1 * n1, a.gd1a, c1 * n1, B, nx, ny, nz, a.shares, st);
   if (s != CLAMP_OK) return s;
   U_TRY(relu_bias_grad<true>(a.gd1a, c1 * n1, a.d1a, c1 * n1, c1, B, n1, dB(10), st));
-  s = conv3_bwd(u, 10, a.cat1, 2 * c1 * n1, a.gd1a, c1 * n1, a.gcat1, 2 * c1 * n1, B, nx, ny, nz, st);
+  s = conv3_bwd(u, 10, a.cat1, 2 * c1 * n1, a.gd1a, c1 * n1, a.gcat1, 2 * c1 * n1, B, nx, ny, nz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // transposed conv up1: u1 = cat1[:, :c1] from d2b
   U_TRY(tconv_dgrad(a.gcat1, 2 * c1 * n1, c1, a.gd2b, c2, W(9), B, nx, ny, nz, bf, st));
@@ -1294,10 +1304,10 @@ extern "C" clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const
   U_TRY(relu_bias_grad<false>(a.gcat1, 2 * c1 * n1, nullptr, 0, c1, B, n1, dB(9), st));
   // decoder level 2
   U_TRY(relu_bias_grad<true>(a.gd2b, c2 * n2, a.d2b, c2 * n2, c2, B, n2, dB(8), st));
-  s = conv3_bwd(u, 8, a.d2a, c2 * n2, a.gd2b, c2 * n2, a.gd2a, c2 * n2, B, hx, hy, hz, st);
+  s = conv3_bwd(u, 8, a.d2a, c2 * n2, a.gd2b, c2 * n2, a.gd2a, c2 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
   U_TRY(relu_bias_grad<true>(a.gd2a, c2 * n2, a.d2a, c2 * n2, c2, B, n2, dB(7), st));
-  s = conv3_bwd(u, 7, a.cat2, 2 * c2 * n2, a.gd2a, c2 * n2, a.gcat2, 2 * c2 * n2, B, hx, hy, hz, st);
+  s = conv3_bwd(u, 7, a.cat2, 2 * c2 * n2, a.gd2a, c2 * n2, a.gcat2, 2 * c2 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // transposed conv up2: u2 = cat2[:, :c2] from btb
   U_TRY(tconv_dgrad(a.gcat2, 2 * c2 * n2, c2, a.gbtb, c3, W(6), B, hx, hy, hz, bf, st));
@@ -1305,30 +1315,30 @@ extern "C" clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const
   U_TRY(relu_bias_grad<false>(a.gcat2, 2 * c2 * n2, nullptr, 0, c2, B, n2, dB(6), st));
   // bottleneck
   U_TRY(relu_bias_grad<true>(a.gbtb, c3 * n3, a.btb, c3 * n3, c3, B, n3, dB(5), st));
-  s = conv3_bwd(u, 5, a.bta, c3 * n3, a.gbtb, c3 * n3, a.gbta, c3 * n3, B, qx, qy, qz, st);
+  s = conv3_bwd(u, 5, a.bta, c3 * n3, a.gbtb, c3 * n3, a.gbta, c3 * n3, B, qx, qy, qz, a.shares, st);
   if (s != CLAMP_OK) return s;
   U_TRY(relu_bias_grad<true>(a.gbta, c3 * n3, a.bta, c3 * n3, c3, B, n3, dB(4), st));
-  s = conv3_bwd(u, 4, a.p2, c2 * n3, a.gbta, c3 * n3, a.gp2, c2 * n3, B, qx, qy, qz, st);
+  s = conv3_bwd(u, 4, a.p2, c2 * n3, a.gbta, c3 * n3, a.gp2, c2 * n3, B, qx, qy, qz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // pool 2 into the skip s2 = cat2[:, c2:] (its gradient already holds the concat path)
   k_pool_bwd<<<pool_grid(hx, hy, hz, c2, B), UT, 0, st>>>(a.gp2, a.arg2, a.gcat2 + c2 * n2, 2 * c2 * n2, c2, B, hx, hy, hz);
   U_TRY(cudaGetLastError());
   // encoder level 2
   U_TRY(relu_bias_grad<true>(a.gcat2 + c2 * n2, 2 * c2 * n2, a.cat2 + c2 * n2, 2 * c2 * n2, c2, B, n2, dB(3), st));
-  s = conv3_bwd(u, 3, a.e2a, c2 * n2, a.gcat2 + c2 * n2, 2 * c2 * n2, a.ge2a, c2 * n2, B, hx, hy, hz, st);
+  s = conv3_bwd(u, 3, a.e2a, c2 * n2, a.gcat2 + c2 * n2, 2 * c2 * n2, a.ge2a, c2 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
   U_TRY(relu_bias_grad<true>(a.ge2a, c2 * n2, a.e2a, c2 * n2, c2, B, n2, dB(2), st));
-  s = conv3_bwd(u, 2, a.p1, c1 * n2, a.ge2a, c2 * n2, a.gp1, c1 * n2, B, hx, hy, hz, st);
+  s = conv3_bwd(u, 2, a.p1, c1 * n2, a.ge2a, c2 * n2, a.gp1, c1 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // pool 1 into the skip s1 = cat1[:, c1:]
   k_pool_bwd<<<pool_grid(nx, ny, nz, c1, B), UT, 0, st>>>(a.gp1, a.arg1, a.gcat1 + c1 * n1, 2 * c1 * n1, c1, B, nx, ny, nz);
   U_TRY(cudaGetLastError());
   // encoder level 1
   U_TRY(relu_bias_grad<true>(a.gcat1 + c1 * n1, 2 * c1 * n1, a.cat1 + c1 * n1, 2 * c1 * n1, c1, B, n1, dB(1), st));
-  s = conv3_bwd(u, 1, a.e1a, c1 * n1, a.gcat1 + c1 * n1, 2 * c1 * n1, a.ge1a, c1 * n1, B, nx, ny, nz, st);
+  s = conv3_bwd(u, 1, a.e1a, c1 * n1, a.gcat1 + c1 * n1, 2 * c1 * n1, a.ge1a, c1 * n1, B, nx, ny, nz, a.shares, st);
   if (s != CLAMP_OK) return s;
   U_TRY(relu_bias_grad<true>(a.ge1a, c1 * n1, a.e1a, c1 * n1, c1, B, n1, dB(0), st));
-  return conv3_bwd(u, 0, x, n1, a.ge1a, c1 * n1, nullptr, 0, B, nx, ny, nz, st);
+  return conv3_bwd(u, 0, x, n1, a.ge1a, c1 * n1, nullptr, 0, B, nx, ny, nz, a.shares, st);
 }
 
 extern "C" clamp_status clamp_unet_adam(clamp_unet* u, float lr, float beta1, float beta2, float eps, int32_t t,
