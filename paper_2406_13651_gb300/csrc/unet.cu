@@ -1240,9 +1240,13 @@ extern "C" clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float*
 // cores) between two lengths of the CUDA cores' FP32 chains:
 //   * below 128 terms a launch more would cost what the tensor cores save (17 against 10 to 17 us), and
 //     the CUDA cores' sums are as exact (64 -> 64 at chains of 85: 4.3e-8 of FP64 against 4.5e-8);
-//   * the longer chains are the less exact of the two, but they are what earlier training runs
-//     followed, and a gradient that leaves them moves by their whole error.
-constexpr long long kTcChainMin = 128, kTcChainFull = 24LL << 10, kTcChainCoarse = 160LL << 10;
+//   * the longer chains are the less exact of the two by far (at 21 k terms 2e-6 of a layer's gradient,
+//     at 79 k 1e-5 to 4e-5; the tensor cores' stay below 1e-7), but they are what earlier training
+//     runs followed, and a gradient that leaves them moves by their whole error.  That error grows
+//     with the length to the power 1.5 to 2, fastest at the full-size level, whose activations carry
+//     the image's background.  Up to the limits it is below 2e-5 of the whole gradient: measured at
+//     most 0.7e-6 at 21 k terms and 1.4e-5 at 41 k there; 9.4e-6 at 79 k and 1.1e-5 at 111 k at the coarser levels.
+constexpr long long kTcChainMin = 128, kTcChainFull = 24LL << 10, kTcChainCoarse = 112LL << 10;
 static clamp_status conv3_bwd(clamp_unet* u, int li, const float* in, long long in_bs, const float* g, long long g_bs,
                               float* din, long long din_bs, int B, int nx, int ny, int nz, float* part, cudaStream_t st) {
   const Layer& L = u->layers[li];
