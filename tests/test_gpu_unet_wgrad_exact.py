@@ -133,6 +133,9 @@ def test_half_size_level(C, shape, B, on_tc):
     child = bf16(2 * d / x.numel()).reshape(B, nz // 2, 2, ny // 2, 2, nx // 2, 2).permute(0, 1, 3, 5, 2, 4, 6).flatten(4)
     g = bf16((child @ torch.from_numpy(sign.T.astype(np.float32)).cuda()).permute(0, 4, 1, 2, 3))   # k times one value, |k| <= 8
     ref = exact_wgrad(shifted(pooled, ch[1]), g)
-    tc, cc = error(run(C, ch, net, layer, x, target, True), ref), error(run(C, ch, net, layer, x, target, False), ref)
-    assert tc < (TC if on_tc else CC), (tc, cc)
-    assert cc < CC, (tc, cc)
+    tc, cc = run(C, ch, net, layer, x, target, True), run(C, ch, net, layer, x, target, False)
+    assert error(cc, ref) < CC
+    if on_tc:
+        assert error(tc, ref) < TC
+    else:   # the same kernel: its three shares in another order at most (a few times 2^-24)
+        assert float((tc - cc).norm() / ref.norm()) < TC
