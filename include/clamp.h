@@ -432,7 +432,8 @@ clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float* y, int32_t
                                 int32_t nz, void* ws, size_t ws_bytes, void* stream);
 /* Forward pass, loss = mean((U-Net(x) - target)^2) over all batch * n outputs, and the
  * gradient of the loss with respect to every parameter (overwrites the gradient buffer).
- * loss: optional DEVICE double. */
+ * loss: optional DEVICE double.  The gradients repeat bit for bit, except the 3x3x3 convs' weights
+ * where they are formed on the CUDA cores (atomics). */
 clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const float* target, int32_t batch, int32_t nx,
                                  int32_t ny, int32_t nz, double* loss, void* ws, size_t ws_bytes, void* stream);
 /* Forward pass and loss = mean((U-Net(x) - target)^2) only (device double); ws as for

@@ -60,4 +60,6 @@ cudaError_t unet_wgrad3_tc(const float* in, long long in_bs, int ci, const float
                            int B, int nx, int ny, int nz, float* part, int* err, cudaStream_t st);
 // Floats `part` needs.
 size_t unet_wgrad3_tc_part(int ci, int co, int B, int nx, int ny, int nz);
+// out[e] = sum over the shares of part[share][e], e < len, always in the same order.
+cudaError_t unet_sum_shares(const float* part, int shares, int len, float* out, cudaStream_t st);
 }  // namespace clamp

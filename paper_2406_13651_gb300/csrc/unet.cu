@@ -318,19 +318,61 @@ __device__ __forceinline__ float block_sum(float v) {
 // Grid of the per-channel reductions below: RC_PER float4 (or values) per thread along a
 // channel plane in x, channels in y, samples in z.  A one-CTA-per-channel reduction leaves
 // 120 to 136 of 152 SMs idle at 16 to 32 channels (3.1 ms for a 0.2 GB tensor at
-// 24 x 64x64x32); here every CTA sums one chunk of a plane and adds it with one atomic.
+// 24 x 64x64x32); here every CTA sums one chunk of a plane into `part`, [channel][sample][chunk], and
+// one launch at the end of the backward pass adds those of every layer in a fixed order.
 constexpr int RC_PER = 4;
 static dim3 chan_grid(long long n, int C, int B) {
   const long long units = n % 4 == 0 ? n / 4 : n;
   return dim3((unsigned)((units + UT * RC_PER - 1) / (UT * RC_PER)), C, std::min(B, 65535));
 }
+static long long chan_parts(long long n, int B) {   // partial sums per channel
+  const dim3 g = chan_grid(n, 1, B);
+  return (long long)g.x * g.z;
+}
+__device__ __forceinline__ long long chan_part(int c) {   // this CTA's
+  return ((long long)c * gridDim.z + blockIdx.z) * gridDim.x + blockIdx.x;
+}
+
+// The sums to take at the end: out[c] = sum of part[c][0 .. per - 1].
+struct ChanSums {
+  static constexpr int MAX = 14;
+  int n = 0, channels[MAX];
+  long long per[MAX];
+  const float* part[MAX];
+  float* out[MAX];
+  float* next;   // free scratch
+  float* add(float* o, int C, long long vox, int B) {
+    float* r = next;
+    out[n] = o;
+    channels[n] = C;
+    per[n] = chan_parts(vox, B);
+    part[n] = r;
+    next += C * per[n++];
+    return r;
+  }
+};
+__global__ void __launch_bounds__(UT) k_chan_sums(ChanSums t) {   // a CTA per channel of every entry
+  int k = 0, c = blockIdx.x;
+  while (c >= t.channels[k]) c -= t.channels[k++];
+  const float* p = t.part[k] + c * t.per[k];
+  float acc = 0.f;
+  for (long long i = threadIdx.x; i < t.per[k]; i += UT) acc += __ldg(p + i);
+  acc = block_sum(acc);
+  if (threadIdx.x == 0) t.out[k][c] = acc;
+}
+static cudaError_t chan_sums(const ChanSums& t, cudaStream_t st) {
+  int total = 0;
+  for (int k = 0; k < t.n; ++k) total += t.channels[k];
+  k_chan_sums<<<total, UT, 0, st>>>(t);
+  return cudaGetLastError();
+}
 
 // g <- g * (y > 0) for a ReLU output y (MASK; sample strides allow concat views) and
-// db[c] += sum_{b, v} g[b][c][v], in one pass.
+// db[c] = sum_{b, v} g[b][c][v], in one pass (partial sums into part).
 template <bool MASK, bool VEC>
 __global__ void __launch_bounds__(UT) k_relu_bias_grad(float* __restrict__ g, long long g_bs,
                                                        const float* __restrict__ y, long long y_bs, int B,
-                                                       long long n, float* __restrict__ db) {
+                                                       long long n, float* __restrict__ part) {
   const int c = blockIdx.y;
   const long long units = VEC ? n / 4 : n;
   const long long u0 = (long long)blockIdx.x * (UT * RC_PER) + threadIdx.x;
@@ -361,16 +403,17 @@ __global__ void __launch_bounds__(UT) k_relu_bias_grad(float* __restrict__ g, lo
     }
   }
   const float s = block_sum(acc);
-  if (threadIdx.x == 0) atomicAdd(&db[c], s);
+  if (threadIdx.x == 0) part[chan_part(c)] = s;
 }
 
 template <bool MASK>
 static cudaError_t relu_bias_grad(float* g, long long g_bs, const float* y, long long y_bs, int C, int B, long long n,
-                                  float* db, cudaStream_t st) {
+                                  float* db, ChanSums& sums, cudaStream_t st) {
+  float* part = sums.add(db, C, n, B);
   if (n % 4 == 0)
-    k_relu_bias_grad<MASK, true><<<chan_grid(n, C, B), UT, 0, st>>>(g, g_bs, y, y_bs, B, n, db);
+    k_relu_bias_grad<MASK, true><<<chan_grid(n, C, B), UT, 0, st>>>(g, g_bs, y, y_bs, B, n, part);
   else
-    k_relu_bias_grad<MASK, false><<<chan_grid(n, C, B), UT, 0, st>>>(g, g_bs, y, y_bs, B, n, db);
+    k_relu_bias_grad<MASK, false><<<chan_grid(n, C, B), UT, 0, st>>>(g, g_bs, y, y_bs, B, n, part);
   return cudaGetLastError();
 }
 
@@ -652,7 +695,7 @@ static cudaError_t tconv_dgrad(const float* dout, long long dout_bs, int co, flo
   return cudaGetLastError();
 }
 
-// dW[ci][co][d] += sum_{b, v} in[b][ci][v] dout[b][co][2v + d]: a product of a [ci][voxel] and a
+// dW[ci][co][d] = sum_{b, v} in[b][ci][v] dout[b][co][2v + d]: a product of a [ci][voxel] and a
 // [voxel][(co, d)] matrix.  A CTA takes 32 input and 16 output channels (32 x 128 sums, 8 x 4 per
 // thread, so three 16-byte shared loads feed 32 FMAs) and a share of the 32-voxel chunks of
 // the samples' flat voxel order, whatever the rows' width; the next chunk's loads are in
@@ -660,12 +703,12 @@ static cudaError_t tconv_dgrad(const float* dout, long long dout_bs, int co, flo
 // 32 -> 16: 43 us of FMAs, 30 us of HBM).  Two sums per thread walked 64-voxel rows, mostly
 // padding at the coarse levels (16 wide: a quarter used): 807 us there and 765 us for 64 -> 32 at
 // half size, now 124 and 63.  A chain is 256 voxels; each is added in FP32 to a second
-// register sum, those with one atomic per sum and CTA.
+// register sum, and a second kernel adds the shares' sums (part[share][ci][co][d]) in a fixed order.
 constexpr int TW_CI = 32, TW_CO = 16, TW_V = 32, TW_NT = 128, TW_CHAIN = 8;   // TW_CHAIN: chunks per chain
 constexpr int TW_XP = TW_CI + 4, TW_GP = TW_CO * 8 + 8;                       // row pitches (floats)
 __global__ void __launch_bounds__(TW_NT, 3) k_tconv_wgrad(const float* __restrict__ in, int ci_n,
                                                           const float* __restrict__ dout, long long dout_bs, int co_n,
-                                                          float* __restrict__ dW, int B, int nx, int ny, int nz, int bf) {
+                                                          float* __restrict__ part, int B, int nx, int ny, int nz, int bf) {
   __shared__ __align__(16) float s_x[2][TW_V][TW_XP];   // [voxel][ci]
   __shared__ __align__(16) float s_g[2][TW_V][TW_GP];   // [voxel][co][d]
   const int ix = nx / 2, iy = ny / 2, iz = nz / 2, in_n = ix * iy * iz;
@@ -760,20 +803,26 @@ __global__ void __launch_bounds__(TW_NT, 3) k_tconv_wgrad(const float* __restric
   for (int i = 0; i < 8; ++i) {
     const int ci = ci0 + 8 * warp + i;
     if (ci >= ci_n) continue;
-    float* d = dW + ((long long)ci * co_n + co) * 8 + 4 * (lane & 1);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) atomicAdd(d + j, sum[i][j]);
+    *reinterpret_cast<float4*>(part + (((long long)blockIdx.x * ci_n + ci) * co_n + co) * 8 + 4 * (lane & 1)) =
+        make_float4(sum[i][0], sum[i][1], sum[i][2], sum[i][3]);
   }
 }
 
-static cudaError_t tconv_wgrad(const float* in, int ci, const float* dout, long long dout_bs, int co, float* dW, int B,
-                               int nx, int ny, int nz, int bf, cudaStream_t st) {
-  const int bi = (ci + TW_CI - 1) / TW_CI, bo = (co + TW_CO - 1) / TW_CO;
+static int tconv_shares(int ci, int co, int B, int nx, int ny, int nz) {
+  const int tiles = ((ci + TW_CI - 1) / TW_CI) * ((co + TW_CO - 1) / TW_CO);
   const long long chunks = (long long)B * (((long long)nx * ny * nz / 8 + TW_V - 1) / TW_V);
-  const long long per = std::max(1, 152 * 3 / (bi * bo));   // one wave of three CTAs per SM
-  k_tconv_wgrad<<<dim3((unsigned)std::min(chunks, per), bi, bo), TW_NT, 0, st>>>(in, ci, dout, dout_bs, co, dW, B, nx, ny,
-                                                                                 nz, bf);
-  return cudaGetLastError();
+  return (int)std::min(chunks, (long long)std::max(1, 152 * 3 / tiles));   // one wave of three CTAs per SM
+}
+static size_t tconv_part(int ci, int co, int B, int nx, int ny, int nz) {   // floats of scratch
+  return (size_t)tconv_shares(ci, co, B, nx, ny, nz) * ci * co * 8;
+}
+static cudaError_t tconv_wgrad(const float* in, int ci, const float* dout, long long dout_bs, int co, float* dW, int B,
+                               int nx, int ny, int nz, int bf, float* part, cudaStream_t st) {
+  const int shares = tconv_shares(ci, co, B, nx, ny, nz);
+  k_tconv_wgrad<<<dim3(shares, (ci + TW_CI - 1) / TW_CI, (co + TW_CO - 1) / TW_CO), TW_NT, 0, st>>>(
+      in, ci, dout, dout_bs, co, part, B, nx, ny, nz, bf);
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : unet_sum_shares(part, shares, ci * co * 8, dW, st);
 }
 
 // 1x1x1 conv to one channel: out[b][v] = bias + sum_c W[c] in[b][c][v], four voxels per thread
@@ -813,14 +862,14 @@ static cudaError_t conv1_fwd(const float* in, int c, const float* W, const float
   return cudaGetLastError();
 }
 // Backward of the 1x1x1 conv and of the ReLU before it, in one pass over the input `in` (the
-// ReLU output): din[b][c][v] = W[c] dout[b][v] where in > 0, else 0; dW[c] += sum in dout;
-// db += sum dout (once, by channel 0's CTAs); dbprev[c] += sum din (the bias of the layer
-// that made `in`).
+// ReLU output): din[b][c][v] = W[c] dout[b][v] where in > 0, else 0; partial sums of dW[c] = sum in dout,
+// db = sum dout (once, by channel 0's CTAs) and dbprev[c] = sum din (the bias of the layer
+// that made `in`) into pw, pb and pp.
 template <bool VEC>
 __global__ void __launch_bounds__(UT) k_conv1_bwd(const float* __restrict__ in, int c_n, const float* __restrict__ dout,
                                                   const float* __restrict__ W, float* __restrict__ din,
-                                                  float* __restrict__ dW, float* __restrict__ db,
-                                                  float* __restrict__ dbprev, int B, long long n, int bf) {
+                                                  float* __restrict__ pw, float* __restrict__ pb,
+                                                  float* __restrict__ pp, int B, long long n, int bf) {
   const int c = blockIdx.y;
   const long long units = VEC ? n / 4 : n;
   const long long u0 = (long long)blockIdx.x * (UT * RC_PER) + threadIdx.x;
@@ -853,9 +902,9 @@ __global__ void __launch_bounds__(UT) k_conv1_bwd(const float* __restrict__ in, 
   sb = block_sum(sb);
   sp = block_sum(sp);
   if (threadIdx.x == 0) {
-    atomicAdd(&dW[c], sw);
-    atomicAdd(&dbprev[c], sp);
-    if (c == 0) atomicAdd(db, sb);
+    pw[chan_part(c)] = sw;
+    pp[chan_part(c)] = sp;
+    if (c == 0) pb[chan_part(0)] = sb;
   }
 }
 
@@ -1037,6 +1086,7 @@ struct Acts {
   unsigned char *arg1, *arg2;
   double* part;
   float* shares;   // partial sums of one weight gradient
+  float* chan;     // partial sums of the biases' and the 1x1 conv's gradients
   size_t bytes;
 };
 
@@ -1065,11 +1115,14 @@ Acts acts_layout(const clamp_unet* u, int B, int nx, int ny, int nz, void* base,
   a.part = reinterpret_cast<double*>(take(2 * 152 * 16));
   if (with_grads) {
     size_t m = 0;
-    if (u->bf)
-      for (const Layer& L : u->layers)
-        if (L.kind == CONV3)
-          m = std::max(m, clamp::unet_wgrad3_tc_part(L.ci, L.co, B, nx / L.level, ny / L.level, nz / L.level));
+    for (const Layer& L : u->layers) {
+      const int lx = nx / L.level, ly = ny / L.level, lz = nz / L.level;
+      if (L.kind == TCONV) m = std::max(m, tconv_part(L.ci, L.co, B, lx, ly, lz));
+      if (L.kind == CONV3 && u->bf) m = std::max(m, clamp::unet_wgrad3_tc_part(L.ci, L.co, B, lx, ly, lz));
+    }
     a.shares = take((long long)m);
+    // five layers' biases at the first two levels, two's at the third; the 1x1 conv's weights and bias
+    a.chan = take((6LL * c1 + 1) * chan_parts(n1, B) + 5LL * c2 * chan_parts(n2, B) + 2LL * c3 * chan_parts(n3, B));
   }
   a.bytes = off;
   return a;
@@ -1293,56 +1346,64 @@ extern "C" clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const
   auto W = [&](int i) { return u->p + u->layers[i].w; };
   auto dB = [&](int i) { return u->g + u->layers[i].b; };
   // output 1x1 conv, the ReLU before it and that layer's bias
-  (n1 % 4 == 0 ? k_conv1_bwd<true> : k_conv1_bwd<false>)<<<chan_grid(n1, c1, B), UT, 0, st>>>(
-      a.d1b, c1, a.gout, W(12), a.gd1b, u->g + u->layers[12].w, dB(12), dB(11), B, n1, bf);
+  ChanSums sums;
+  sums.next = a.chan;
+  float* pw = sums.add(u->g + u->layers[12].w, c1, n1, B);
+  float* pb = sums.add(dB(12), 1, n1, B);
+  float* pp = sums.add(dB(11), c1, n1, B);
+  (n1 % 4 == 0 ? k_conv1_bwd<true> : k_conv1_bwd<false>)<<<chan_grid(n1, c1, B), UT, 0, st>>>(a.d1b, c1, a.gout, W(12), a.gd1b,
+                                                                                              pw, pb, pp, B, n1, bf);
   U_TRY(cudaGetLastError());
   // decoder level 1
   s = conv3_bwd(u, 11, a.d1a, c1 * n1, a.gd1b, c1 * n1, a.gd1a, c1 * n1, B, nx, ny, nz, a.shares, st);
   if (s != CLAMP_OK) return s;
-  U_TRY(relu_bias_grad<true>(a.gd1a, c1 * n1, a.d1a, c1 * n1, c1, B, n1, dB(10), st));
+  U_TRY(relu_bias_grad<true>(a.gd1a, c1 * n1, a.d1a, c1 * n1, c1, B, n1, dB(10), sums, st));
   s = conv3_bwd(u, 10, a.cat1, 2 * c1 * n1, a.gd1a, c1 * n1, a.gcat1, 2 * c1 * n1, B, nx, ny, nz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // transposed conv up1: u1 = cat1[:, :c1] from d2b
   U_TRY(tconv_dgrad(a.gcat1, 2 * c1 * n1, c1, a.gd2b, c2, W(9), B, nx, ny, nz, bf, st));
-  U_TRY(tconv_wgrad(a.d2b, c2, a.gcat1, 2 * c1 * n1, c1, u->g + u->layers[9].w, B, nx, ny, nz, bf, st));
-  U_TRY(relu_bias_grad<false>(a.gcat1, 2 * c1 * n1, nullptr, 0, c1, B, n1, dB(9), st));
+  U_TRY(tconv_wgrad(a.d2b, c2, a.gcat1, 2 * c1 * n1, c1, u->g + u->layers[9].w, B, nx, ny, nz, bf, a.shares, st));
+  U_TRY(relu_bias_grad<false>(a.gcat1, 2 * c1 * n1, nullptr, 0, c1, B, n1, dB(9), sums, st));
   // decoder level 2
-  U_TRY(relu_bias_grad<true>(a.gd2b, c2 * n2, a.d2b, c2 * n2, c2, B, n2, dB(8), st));
+  U_TRY(relu_bias_grad<true>(a.gd2b, c2 * n2, a.d2b, c2 * n2, c2, B, n2, dB(8), sums, st));
   s = conv3_bwd(u, 8, a.d2a, c2 * n2, a.gd2b, c2 * n2, a.gd2a, c2 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
-  U_TRY(relu_bias_grad<true>(a.gd2a, c2 * n2, a.d2a, c2 * n2, c2, B, n2, dB(7), st));
+  U_TRY(relu_bias_grad<true>(a.gd2a, c2 * n2, a.d2a, c2 * n2, c2, B, n2, dB(7), sums, st));
   s = conv3_bwd(u, 7, a.cat2, 2 * c2 * n2, a.gd2a, c2 * n2, a.gcat2, 2 * c2 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // transposed conv up2: u2 = cat2[:, :c2] from btb
   U_TRY(tconv_dgrad(a.gcat2, 2 * c2 * n2, c2, a.gbtb, c3, W(6), B, hx, hy, hz, bf, st));
-  U_TRY(tconv_wgrad(a.btb, c3, a.gcat2, 2 * c2 * n2, c2, u->g + u->layers[6].w, B, hx, hy, hz, bf, st));
-  U_TRY(relu_bias_grad<false>(a.gcat2, 2 * c2 * n2, nullptr, 0, c2, B, n2, dB(6), st));
+  U_TRY(tconv_wgrad(a.btb, c3, a.gcat2, 2 * c2 * n2, c2, u->g + u->layers[6].w, B, hx, hy, hz, bf, a.shares, st));
+  U_TRY(relu_bias_grad<false>(a.gcat2, 2 * c2 * n2, nullptr, 0, c2, B, n2, dB(6), sums, st));
   // bottleneck
-  U_TRY(relu_bias_grad<true>(a.gbtb, c3 * n3, a.btb, c3 * n3, c3, B, n3, dB(5), st));
+  U_TRY(relu_bias_grad<true>(a.gbtb, c3 * n3, a.btb, c3 * n3, c3, B, n3, dB(5), sums, st));
   s = conv3_bwd(u, 5, a.bta, c3 * n3, a.gbtb, c3 * n3, a.gbta, c3 * n3, B, qx, qy, qz, a.shares, st);
   if (s != CLAMP_OK) return s;
-  U_TRY(relu_bias_grad<true>(a.gbta, c3 * n3, a.bta, c3 * n3, c3, B, n3, dB(4), st));
+  U_TRY(relu_bias_grad<true>(a.gbta, c3 * n3, a.bta, c3 * n3, c3, B, n3, dB(4), sums, st));
   s = conv3_bwd(u, 4, a.p2, c2 * n3, a.gbta, c3 * n3, a.gp2, c2 * n3, B, qx, qy, qz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // pool 2 into the skip s2 = cat2[:, c2:] (its gradient already holds the concat path)
   k_pool_bwd<<<pool_grid(hx, hy, hz, c2, B), UT, 0, st>>>(a.gp2, a.arg2, a.gcat2 + c2 * n2, 2 * c2 * n2, c2, B, hx, hy, hz);
   U_TRY(cudaGetLastError());
   // encoder level 2
-  U_TRY(relu_bias_grad<true>(a.gcat2 + c2 * n2, 2 * c2 * n2, a.cat2 + c2 * n2, 2 * c2 * n2, c2, B, n2, dB(3), st));
+  U_TRY(relu_bias_grad<true>(a.gcat2 + c2 * n2, 2 * c2 * n2, a.cat2 + c2 * n2, 2 * c2 * n2, c2, B, n2, dB(3), sums, st));
   s = conv3_bwd(u, 3, a.e2a, c2 * n2, a.gcat2 + c2 * n2, 2 * c2 * n2, a.ge2a, c2 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
-  U_TRY(relu_bias_grad<true>(a.ge2a, c2 * n2, a.e2a, c2 * n2, c2, B, n2, dB(2), st));
+  U_TRY(relu_bias_grad<true>(a.ge2a, c2 * n2, a.e2a, c2 * n2, c2, B, n2, dB(2), sums, st));
   s = conv3_bwd(u, 2, a.p1, c1 * n2, a.ge2a, c2 * n2, a.gp1, c1 * n2, B, hx, hy, hz, a.shares, st);
   if (s != CLAMP_OK) return s;
   // pool 1 into the skip s1 = cat1[:, c1:]
   k_pool_bwd<<<pool_grid(nx, ny, nz, c1, B), UT, 0, st>>>(a.gp1, a.arg1, a.gcat1 + c1 * n1, 2 * c1 * n1, c1, B, nx, ny, nz);
   U_TRY(cudaGetLastError());
   // encoder level 1
-  U_TRY(relu_bias_grad<true>(a.gcat1 + c1 * n1, 2 * c1 * n1, a.cat1 + c1 * n1, 2 * c1 * n1, c1, B, n1, dB(1), st));
+  U_TRY(relu_bias_grad<true>(a.gcat1 + c1 * n1, 2 * c1 * n1, a.cat1 + c1 * n1, 2 * c1 * n1, c1, B, n1, dB(1), sums, st));
   s = conv3_bwd(u, 1, a.e1a, c1 * n1, a.gcat1 + c1 * n1, 2 * c1 * n1, a.ge1a, c1 * n1, B, nx, ny, nz, a.shares, st);
   if (s != CLAMP_OK) return s;
-  U_TRY(relu_bias_grad<true>(a.ge1a, c1 * n1, a.e1a, c1 * n1, c1, B, n1, dB(0), st));
-  return conv3_bwd(u, 0, x, n1, a.ge1a, c1 * n1, nullptr, 0, B, nx, ny, nz, a.shares, st);
+  U_TRY(relu_bias_grad<true>(a.ge1a, c1 * n1, a.e1a, c1 * n1, c1, B, n1, dB(0), sums, st));
+  s = conv3_bwd(u, 0, x, n1, a.ge1a, c1 * n1, nullptr, 0, B, nx, ny, nz, a.shares, st);
+  if (s != CLAMP_OK) return s;
+  U_TRY(chan_sums(sums, st));
+  return CLAMP_OK;
 }
 
 extern "C" clamp_status clamp_unet_adam(clamp_unet* u, float lr, float beta1, float beta2, float eps, int32_t t,

@@ -327,6 +327,9 @@ __global__ void __launch_bounds__(32 * SH_G) k_sum_shares(const float* __restric
   if (i >= 0) out[i] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
 }
 
+struct Identity {
+  __device__ long long operator()(int, int e) const { return e; }
+};
 // Element e ([dz][dy][ci][dx][co]) of channel-chunk pair `pair` in dW[co][ci][27], or -1.
 template <int CO, int NCH>
 struct WgMap {
@@ -374,6 +377,12 @@ static size_t part_floats(int ci, int co, int B, int nx, int ny, int nz) {
 }
 
 }  // namespace unet_wg
+
+cudaError_t unet_sum_shares(const float* part, int shares, int len, float* out, cudaStream_t st) {
+  using namespace unet_wg;
+  k_sum_shares<<<(len + 31) / 32, 32 * SH_G, 0, st>>>(part, shares, len, out, Identity{});
+  return cudaGetLastError();
+}
 
 size_t unet_wgrad3_tc_part(int ci, int co, int B, int nx, int ny, int nz) {
   using namespace unet_wg;
