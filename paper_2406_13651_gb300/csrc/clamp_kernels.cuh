@@ -112,7 +112,9 @@ inline cudaError_t launch_after(void (*k)(P...), dim3 grid, unsigned threads, si
   cfg.stream = st;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, P(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, P(args)...);
+  if (e != cudaSuccess) cudaGetLastError();   // reported here, not by the next call's check
+  return e;
 }
 #ifdef __CUDACC__
 // First statement of a kernel launched so: lets the next kernel's CTAs be set up, then waits until
