@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(RCol<N>::THREADS, RCol<N>::MINB) k_band_z_inv(
   const int col = threadIdx.x % BC, j = threadIdx.x / BC;
   const int s = blockIdx.x * BC + col, l = blockIdx.y;
   const long long cbase = (long long)l * N * a.t.nSp + s;   // compact [l][kz][s]
-  const float gp = a.gamma_prev ? __ldg(&a.gamma_prev[l]) : 0.0f;
+  const float gp = a.gamma_prev ? a.gamma_prev[l] : 0.0f;
   const bool valid = s < a.t.nS;   // padding columns hold stale values: read as zero
   const bool step = valid && a.gamma_prev;
   const float pup = __ldg(&a.t.s_pup[s]);

@@ -980,16 +980,20 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
     // two looks ahead in flight: slot a holds look l + 1, slot b look l + 2
     float2 w_n = Wi[vp], r_n = Ri[vp];
     float4 m_n = make_float4(0.f, 0.f, 0.f, 0.f), d_n = m_n;
+    [[maybe_unused]] float g_n = 0.f;
     if constexpr (PROX) {
+      if (!c.closed_mu) g_n = c.gamma[0];
       m_n = __ldcs(&MUi[vp]);
       d_n = __ldcs(&Di[vp]);
     }
     float2 w_a = w_n, r_a = r_n;
     float4 m_a = m_n, d_a = d_n;
+    [[maybe_unused]] float g_a = 0.f;
     if (L > 1) {
       w_a = Wi[n2 + vp];
       r_a = Ri[n2 + vp];
       if constexpr (PROX) {
+        if (!c.closed_mu) g_a = c.gamma[1];
         m_a = __ldcs(&MUi[n2 + vp]);
         d_a = __ldcs(&Di[n2 + vp]);
       }
@@ -1000,14 +1004,17 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
       const float2 wl = w_n, rp = r_n;
       [[maybe_unused]] float4 m = m_n;
       [[maybe_unused]] const float4 dd = d_n;
+      [[maybe_unused]] const float gm = g_n;
       w_n = w_a;
       r_n = r_a;
       m_n = m_a;
       d_n = d_a;
+      g_n = g_a;
       if (l + 2 < L && CLAMP_IN_BOUNDS(i + 2 * n2, look_ext, 201)) {
         w_a = Wi[i + 2 * n2];
         r_a = Ri[i + 2 * n2];
         if constexpr (PROX) {
+          if (!c.closed_mu) g_a = c.gamma[l + 2];
           m_a = __ldcs(&MUi[i + 2 * n2]);
           d_a = __ldcs(&Di[i + 2 * n2]);
         }
@@ -1027,7 +1034,6 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
           const float f0 = 1.0f / (1.0f + c.nv / (rp.x + c.nv)), f1 = 1.0f / (1.0f + c.nv / (rp.y + c.nv));
           m = make_float4(dd.x * f0, dd.y * f0, dd.z * f1, dd.w * f1);
         } else {
-          const float gm = __ldg(&c.gamma[l]);
           m = make_float4(fmaf(gm, dd.x, m.x), fmaf(gm, dd.y, m.y), fmaf(gm, dd.z, m.z), fmaf(gm, dd.w, m.w));
         }
         const bool in_look = CLAMP_IN_BOUNDS(i, look_ext, 202);

@@ -119,6 +119,10 @@ inline cudaError_t launch_after(void (*k)(P...), dim3 grid, unsigned threads, si
 #ifdef __CUDACC__
 // First statement of a kernel launched so: lets the next kernel's CTAs be set up, then waits until
 // the previous kernel is complete and its writes are visible (no wait if it was launched plainly).
+// The kernel may be resident while those before it still write, so what a kernel of the chain writes (the
+// step gamma, say) is not read through __ldg, whose data has to be read-only for as long as the
+// kernel is resident.  The pupil, the window, the twiddles and the support's tables may be: the kernel that
+// builds the tables is launched plainly and lets nothing start before it has finished.
 __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.launch_dependents;");
   asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -1,5 +1,6 @@
 """Programmatic dependent launches: their error handling, on the CPU."""
 import os
+import re
 import shutil
 import subprocess
 
@@ -52,3 +53,32 @@ def test_refused_launch_is_reported_once(tmp_path):
     assert r.returncode == 0, r.stderr
     out = subprocess.run([exe], capture_output=True, text=True, timeout=120)
     assert out.stdout.split() == ["9", "0", "0", "0"], out.stdout   # the refusal, and no error left for the next call
+
+
+# What a kernel of such a chain may read through the non-coherent path (__ldg): data that nothing in the
+# chain writes.  The kernel may be resident while the one before it still runs, and only what is read-only for as
+# long as it is resident may be read so.
+READ_ONLY = ("a.t.", "a.window", "c.window", "tw")
+
+
+def _bodies(text):
+    """Bodies of the functions that call after_previous()."""
+    at = 0
+    while (at := text.find("  after_previous();", at)) >= 0:
+        depth, end = 1, at
+        while depth:
+            depth += {"{": 1, "}": -1}.get(text[end], 0)
+            end += 1
+        yield text[at:end]
+        at = end
+
+
+def test_dependent_kernels_read_the_chains_data_coherently():
+    seen = 0
+    for name in sorted(os.listdir(os.path.join(PKG, "csrc"))):
+        with open(os.path.join(PKG, "csrc", name)) as f:
+            for body in _bodies(f.read()):
+                seen += 1
+                for arg in re.findall(r"__ldg\(\s*&?\s*([\w.\->]+)", body):
+                    assert arg.startswith(READ_ONLY), (name, arg)
+    assert seen >= 5   # the band passes and the fused pass
