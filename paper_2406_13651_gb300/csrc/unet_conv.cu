@@ -235,9 +235,11 @@ static cudaError_t by_voxels(long long outputs, int co, A... a) {
 }
 
 template <bool BF, typename... A>
-static cudaError_t by_width(long long outputs, int nx, int co, A... a) {
+static cudaError_t by_width(long long outputs, int nx, int ny, int co, A... a) {
   if (nx <= 8) return by_channels<8, 4, BF>(co, a...);
-  if ((nx + 15) / 16 % 2) return by_voxels<16, BF>(outputs, co, a...);   // 32-wide tiles would leave half a tile unused
+  // 16 wide where 32-wide tiles would leave half a tile unused, and above the height at which those of 4 rows
+  // (64 channels) are more than a grid's y extent holds
+  if ((nx + 15) / 16 % 2 || ny > 4 * 65535) return by_voxels<16, BF>(outputs, co, a...);
   return by_voxels<32, BF>(outputs, co, a...);
 }
 
@@ -247,8 +249,8 @@ cudaError_t unet_conv3_cc(bool bf, const float* in, long long in_bs, int ci, flo
                           const float* W, const float* bias, bool relu, int B, int nx, int ny, int nz,
                           cudaStream_t st) {
   const long long outputs = (long long)B * nx * ny * nz * co;
-  return bf ? unet_cc::by_width<true>(outputs, nx, co, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st)
-            : unet_cc::by_width<false>(outputs, nx, co, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st);
+  return bf ? unet_cc::by_width<true>(outputs, nx, ny, co, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st)
+            : unet_cc::by_width<false>(outputs, nx, ny, co, in, in_bs, ci, out, out_bs, co, W, bias, relu, B, nx, ny, nz, st);
 }
 
 }  // namespace clamp
