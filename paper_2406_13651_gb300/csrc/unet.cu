@@ -1236,6 +1236,13 @@ static bool on_unet_device(const clamp_unet* u, const char* where) {
   return true;
 }
 
+// The kernels access the workspace 16 bytes at a time.
+static clamp_status check_unet_ws(const void* ws, size_t have, size_t need, const char* where) {
+  if (!ws || have < need) return api_fail(CLAMP_ENOMEM, "%s: workspace too small", where);
+  if ((uintptr_t)ws & 255) return api_fail(CLAMP_EINVAL, "%s: workspace must be 256-byte aligned", where);
+  return CLAMP_OK;
+}
+
 #define U_TRY(x)                                                                       \
   do {                                                                                 \
     cudaError_t _e = (x);                                                              \
@@ -1277,7 +1284,7 @@ extern "C" clamp_status clamp_unet_forward(clamp_unet* u, const float* x, float*
   if (!unet_shape_ok(batch, nx, ny, nz))
     return api_fail(CLAMP_EINVAL, "clamp_unet_forward: nx, ny, nz must be multiples of 4");
   const Acts a = acts_layout(u, batch, nx, ny, nz, ws, false);
-  if (!ws || ws_bytes < a.bytes) return api_fail(CLAMP_ENOMEM, "clamp_unet_forward: workspace too small");
+  if (const clamp_status w = check_unet_ws(ws, ws_bytes, a.bytes, "clamp_unet_forward")) return w;
   cudaStream_t st = (cudaStream_t)stream;
   clamp_status s = unet_forward(u, x, batch, nx, ny, nz, a, st);
   if (s != CLAMP_OK) return s;
@@ -1326,7 +1333,7 @@ extern "C" clamp_status clamp_unet_backward(clamp_unet* u, const float* x, const
   if (!unet_shape_ok(batch, nx, ny, nz))
     return api_fail(CLAMP_EINVAL, "clamp_unet_backward: nx, ny, nz must be multiples of 4");
   const Acts a = acts_layout(u, batch, nx, ny, nz, ws, true);
-  if (!ws || ws_bytes < a.bytes) return api_fail(CLAMP_ENOMEM, "clamp_unet_backward: workspace too small");
+  if (const clamp_status w = check_unet_ws(ws, ws_bytes, a.bytes, "clamp_unet_backward")) return w;
   cudaStream_t st = (cudaStream_t)stream;
   const int bf = u->bf;
   const int B = batch, c1 = u->c1, c2 = u->c2, c3 = u->c3;
@@ -1451,7 +1458,7 @@ extern "C" clamp_status clamp_unet_warm_start(clamp_unet* u, int32_t nx, int32_t
   if (!unet_shape_ok(1, nx, ny, nz))
     return api_fail(CLAMP_EINVAL, "clamp_unet_warm_start: nx, ny, nz must be multiples of 4");
   const Acts a = acts_layout(u, 1, nx, ny, nz, ws, false);
-  if (!ws || ws_bytes < a.bytes) return api_fail(CLAMP_ENOMEM, "clamp_unet_warm_start: workspace too small");
+  if (const clamp_status w = check_unet_ws(ws, ws_bytes, a.bytes, "clamp_unet_warm_start")) return w;
   cudaStream_t st = (cudaStream_t)stream;
   const long long n = (long long)nx * ny * nz;
   // four CTAs per SM: every CTA of the two element-wise passes adds all the partial sums
@@ -1479,7 +1486,7 @@ extern "C" clamp_status clamp_unet_loss(clamp_unet* u, const float* x, const flo
   if (!unet_shape_ok(batch, nx, ny, nz))
     return api_fail(CLAMP_EINVAL, "clamp_unet_loss: nx, ny, nz must be multiples of 4");
   const Acts a = acts_layout(u, batch, nx, ny, nz, ws, true);   // the loss gradient goes to gout
-  if (!ws || ws_bytes < a.bytes) return api_fail(CLAMP_ENOMEM, "clamp_unet_loss: workspace too small");
+  if (const clamp_status w = check_unet_ws(ws, ws_bytes, a.bytes, "clamp_unet_loss")) return w;
   cudaStream_t st = (cudaStream_t)stream;
   clamp_status s = unet_forward(u, x, batch, nx, ny, nz, a, st);
   if (s != CLAMP_OK) return s;
