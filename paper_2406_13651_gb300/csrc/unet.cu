@@ -9,6 +9,7 @@
 #include "../../include/clamp.h"
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
+#include "exact_sum.cuh"
 
 #include <cuda_bf16.h>
 #include <math.h>
@@ -982,9 +983,7 @@ __global__ void __launch_bounds__(NORM_T) k_sample_norm(const float* __restrict_
   }
 }
 
-// Partial sums of x (one per CTA, FP64).  Four elements are first added without error into a FP32 head
-// and tail (two-sum), so FP64, of which an SM does two a clock, adds two values per four
-// elements instead of converting and adding four: 43 -> 21 us at 256x256x128.
+// Partial sums of x (one per CTA, FP64), four elements at a time (exact_sum.cuh): 43 -> 22 us at 256x256x128.
 template <bool VEC>
 __global__ void __launch_bounds__(UT) k_sum_part(const float* __restrict__ x, long long n, double* __restrict__ part) {
   double acc = 0.0;
@@ -992,19 +991,7 @@ __global__ void __launch_bounds__(UT) k_sum_part(const float* __restrict__ x, lo
   if constexpr (VEC) {
     for (long long i = t0; i < n / 4; i += step) {
       const float4 v = __ldg(reinterpret_cast<const float4*>(x) + i);
-      auto two_sum = [](float a, float b, float& e) {
-        const float t = a + b, bp = t - a;
-        e = (a - (t - bp)) + (b - bp);
-        return t;
-      };
-      float e0, e1, e2;
-      const float s0 = two_sum(v.x, v.y, e0), s1 = two_sum(v.z, v.w, e1), t = two_sum(s0, s1, e2);
-      if (isfinite(t)) {
-        acc += (double)t;
-        acc += (double)(e2 + (e0 + e1));   // rounded at 2^-24 of the rounding errors
-      } else {   // a value that is not finite, or a sum beyond FP32
-        acc += ((double)v.x + v.y) + ((double)v.z + v.w);
-      }
+      add_four(acc, v.x, v.y, v.z, v.w);
     }
   } else {
     for (long long i = t0; i < n; i += step) acc += x[i];
