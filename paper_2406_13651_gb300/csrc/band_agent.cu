@@ -125,9 +125,7 @@ __global__ void __launch_bounds__(1024) k_band_tables(const float* __restrict__ 
     const int b = s_first[tid >> 5] + __popc(any & below);
     const bool in_band = any >> lane & 1u;
     t.bpos[tid] = in_band ? b : -1;
-    if (in_band) t.bx[b] = tid;
   }
-  for (int b = t.nbx + tid; b < t.nbxp; b += (int)blockDim.x) t.bx[b] = -1;
   __syncthreads();
   for (int ky = warp; ky < ny; ky += 32) {
     int* row = t.sidx + (long long)ky * t.nbxp;
@@ -559,7 +557,7 @@ BandShape band_shape(const float* pupil_host, int nx, int ny, double* sum_sq) {
 size_t band_table_bytes(const BandShape& b, int nx, int ny) {
   auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
   return al(sizeof(int) * (size_t)ny * b.nbxp) + al(sizeof(int) * (size_t)b.nSp) + al(sizeof(float) * (size_t)b.nSp) +
-         al(sizeof(int) * (size_t)b.nbxp) + al(sizeof(int) * (size_t)nx);
+         al(sizeof(int) * (size_t)nx);
 }
 
 BandTables band_tables_at(const BandShape& b, int nx, int ny, void* base) {
@@ -576,8 +574,6 @@ BandTables band_tables_at(const BandShape& b, int nx, int ny, void* base) {
   p += al(sizeof(int) * (size_t)b.nSp);
   t.s_pup = reinterpret_cast<float*>(p);
   p += al(sizeof(float) * (size_t)b.nSp);
-  t.bx = reinterpret_cast<int*>(p);
-  p += al(sizeof(int) * (size_t)b.nbxp);
   t.bpos = reinterpret_cast<int*>(p);
   return t;
 }

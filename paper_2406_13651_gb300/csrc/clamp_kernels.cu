@@ -391,7 +391,6 @@ struct ColArgs {
   long long stride;    // element stride of the FFT axis
   long long slab;      // element stride of grid.y (fixed index of the other axis)
   int nx;
-  int zaxis;           // 1 when the FFT axis is z (aperture epilogue / prologue)
 };
 
 // Launch variant 0: 16 adjacent lines per CTA, points in registers, one exchange (fft_reg.cuh).
@@ -525,7 +524,6 @@ static ColArgs col_args(const Geom& g, bool zaxis) {
   ColArgs a{};
   a.n = g.n;
   a.nx = g.nx;
-  a.zaxis = zaxis;
   if (zaxis) {
     a.stride = (long long)g.nx * g.ny;
     a.slab = g.nx;
@@ -976,7 +974,6 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
   [[maybe_unused]] float acc[2] = {0.f, 0.f};
   for (long long vp = (long long)blockIdx.x * NT + threadIdx.x; vp < n2; vp += (long long)gridDim.x * NT) {
     [[maybe_unused]] CSum wb0, xb0, wb1, xb1;
-    bool bad = false;
     // two looks ahead in flight: slot a holds look l + 1, slot b look l + 2
     float2 w_n = Wi[vp], r_n = Ri[vp];
     float4 m_n = make_float4(0.f, 0.f, 0.f, 0.f), d_n = m_n;
@@ -1044,10 +1041,7 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
         rn = make_float2(prox_quad(wl.x, rp.x, K0, c.prox_var, c.inv_prox_var, c.beta, c.inv_beta),
                          prox_quad(wl.y, rp.y, K1, c.prox_var, c.inv_prox_var, c.beta, c.inv_beta));
         if (in_look) Ro[i] = rn;
-        // K covers mu: the prox's clip would hide a NaN there.  Without the Mann step's sums below,
-        // products with zero: NaN iff some K or r is not finite
-        if constexpr (MACE) kacc += K0 + K1;
-        else kacc = fmaf(K0, 0.f, fmaf(K1, 0.f, fmaf(rn.x, 0.f, fmaf(rn.y, 0.f, kacc))));
+        kacc += K0 + K1;   // K covers mu: the prox's clip would hide a NaN there
       }
       if constexpr (MACE) {
         wb0.add(c.ups_look * wl.x);
@@ -1056,7 +1050,6 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
         xb1.add(c.ups_look * (2.0f * rn.y - wl.y));
       }
     }
-    if constexpr (PROX) bad |= !isfinite(kacc);
     if constexpr (MACE) {
       const long long ip = (long long)L * n2 + vp;
       const float2 rpr = Ri[ip], wpr = Wi[ip];
@@ -1088,13 +1081,16 @@ __global__ void __launch_bounds__(NT) k_pass_c_pair(Geom g, PassC c) {
       }
       const float wbn0 = wn0.get(), wbn1 = wn1.get();
       reinterpret_cast<float2*>(c.wbar)[vp] = make_float2(wbn0, wbn1);
-      // a non-finite r, w or K of any look reaches these sums (NaN and Inf propagate through
-      // the adds), so one check per voxel pair replaces one per value
-      bad |= !isfinite(x0) || !isfinite(x1) || !isfinite(w0) || !isfinite(w1) || !isfinite(wbn0) || !isfinite(wbn1);
+      if constexpr (PROX) {
+        // a non-finite r, w or K of any look reaches these sums (NaN and Inf propagate through
+        // the adds), so one check per voxel pair replaces one per value
+        const bool bad = !isfinite(kacc) || !isfinite(x0) || !isfinite(x1) || !isfinite(w0) || !isfinite(w1) ||
+                         !isfinite(wbn0) || !isfinite(wbn1);
+        if (bad && c.err) atomicOr(c.err, 1);
+      }
       acc[0] += num;
       acc[1] += (float)(L + 1) * (w0 * w0 + w1 * w1);
     }
-    if (bad && c.err) atomicOr(c.err, 1);
   }
   if constexpr (MACE) {
     double* const outs[2] = {c.part_num, c.part_den};

@@ -140,7 +140,6 @@ struct BandTables {
   int* sidx;      // [ny][nbxp] support index of (ky, band column b), or -1
   int* s_kykx;    // [nSp] ky * nx + kx of support column s (padding: 0)
   float* s_pup;   // [nSp] pupil value of support column s (padding: 0)
-  int* bx;        // [nbxp] kx of band column b (padding: -1)
   int* bpos;      // [nx] band column of kx, or -1
 };
 struct BandArgs {
@@ -215,7 +214,7 @@ struct PassC {
   float ups_look, ups_prior, rho;
   double* part_num;  // CE partials (MACE variants)
   double* part_den;
-  int* err;          // device error word (non-finite)
+  int* err;          // device error word (non-finite) of the fused pass
   int exact_prox;    // 1: exact cubic-root prox instead of the quadratic-surrogate step
   int closed_mu;     // 1: mu = d / (1 + sigma_w^2 / (r' + sigma_w^2)) with d holding F^H y (no aperture)
   // Fused pass: the last CTA to finish adds up the iteration's residuals (null: not asked for).
