@@ -32,6 +32,7 @@
 #include "../../include/clamp.h"
 #include "clamp_kernels.cuh"
 #include "denoise.cuh"
+#include "packed.cuh"
 #include "tc_core.cuh"
 
 #include <cuda_bf16.h>
@@ -115,10 +116,6 @@ struct TcCfg {
   static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-  const __nv_bfloat16 lo = __float2bfloat16_rn(a), hi = __float2bfloat16_rn(b);
-  return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
-}
 // Round to the nearest TF32 value (10 explicit mantissa bits), ties to even.
 __device__ __forceinline__ float tf32_rn(float x) {
   uint32_t u = __float_as_uint(x);
@@ -395,8 +392,8 @@ __global__ void __launch_bounds__(TC_NT, TcKind<KIND>::MIN_CTAS)
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = fmaxf(v[i] + __ldg(&bias[col + i]), 0.f);
           s_halo[(mt * G + col / 8) * 128 + 32 * q + lane] =
-              make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]),
-                         pack_bf16x2(v[6], v[7]));
+              make_uint4(bf16x2(v[0], v[1]), bf16x2(v[2], v[3]), bf16x2(v[4], v[5]),
+                         bf16x2(v[6], v[7]));
         }
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -482,10 +479,10 @@ __global__ void __launch_bounds__(TC_NT, TcKind<KIND>::MIN_CTAS)
         for (int i = 0; i < 8; ++i) v[i] = fmaxf(v[i] + __ldg(&bias[col + i]), 0.f);
         if constexpr (KIND == TC_BF16) {
           uint4 o;
-          o.x = pack_bf16x2(v[0], v[1]);
-          o.y = pack_bf16x2(v[2], v[3]);
-          o.z = pack_bf16x2(v[4], v[5]);
-          o.w = pack_bf16x2(v[6], v[7]);
+          o.x = bf16x2(v[0], v[1]);
+          o.y = bf16x2(v[2], v[3]);
+          o.z = bf16x2(v[4], v[5]);
+          o.w = bf16x2(v[6], v[7]);
           if (CLAMP_IN_BOUNDS((long long)(col / 8) * n + vox, out_ext, 306)) out_act[(long long)(col / 8) * n + vox] = o;
         } else {
           float4* o4 = reinterpret_cast<float4*>(out_act);
@@ -713,10 +710,10 @@ __device__ __forceinline__ void store_first(uint4* out, long long n, long long v
 #pragma unroll
     for (int g = 0; g < C / 8; ++g) {
       uint4 o;
-      o.x = pack_bf16x2(acc[8 * g + 0], acc[8 * g + 1]);
-      o.y = pack_bf16x2(acc[8 * g + 2], acc[8 * g + 3]);
-      o.z = pack_bf16x2(acc[8 * g + 4], acc[8 * g + 5]);
-      o.w = pack_bf16x2(acc[8 * g + 6], acc[8 * g + 7]);
+      o.x = bf16x2(acc[8 * g + 0], acc[8 * g + 1]);
+      o.y = bf16x2(acc[8 * g + 2], acc[8 * g + 3]);
+      o.z = bf16x2(acc[8 * g + 4], acc[8 * g + 5]);
+      o.w = bf16x2(acc[8 * g + 6], acc[8 * g + 7]);
       out[(long long)g * n + v] = o;
     }
   } else {
@@ -1199,10 +1196,10 @@ __global__ void __launch_bounds__(TC_NT) k_conv_first_tc(const float* __restrict
 #pragma unroll
           for (int i = 0; i < 8; ++i) v[i] = fmaxf(v[i] + __ldg(&bias[col + i]), 0.f);
           uint4 o;
-          o.x = pack_bf16x2(v[0], v[1]);
-          o.y = pack_bf16x2(v[2], v[3]);
-          o.z = pack_bf16x2(v[4], v[5]);
-          o.w = pack_bf16x2(v[6], v[7]);
+          o.x = bf16x2(v[0], v[1]);
+          o.y = bf16x2(v[2], v[3]);
+          o.z = bf16x2(v[4], v[5]);
+          o.w = bf16x2(v[6], v[7]);
           if (CLAMP_IN_BOUNDS((long long)(col / 8) * n + vox, (long long)(C / 8) * n, 312))
             out[(long long)(col / 8) * n + vox] = o;
         }

@@ -10,6 +10,7 @@
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
 #include "exact_sum.cuh"
+#include "packed.cuh"
 
 #include <cuda_bf16.h>
 #include <math.h>
@@ -26,23 +27,6 @@ constexpr int UT = 256;
 // BF16 mode: an operand rounded to bfloat16 (round to nearest even) and widened back.
 __device__ __forceinline__ float opr(float x, int bf) {
   return bf ? __bfloat162float(__float2bfloat16_rn(x)) : x;
-}
-
-// Two packed FP32 values; fma2 rounds each half as fmaf does.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(unsigned long long v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
 }
 
 enum LayerKind { CONV3 = 0, TCONV = 1, CONV1 = 2 };
@@ -486,9 +470,6 @@ constexpr int TF_CO = 16;
 static size_t tconv_fwd_smem(int ci, int vpt, int nbuf) { return sizeof(float) * (size_t)ci * (TF_CO * 8 + nbuf * 64 * vpt); }
 __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 template <int VPT>
 __global__ void __launch_bounds__(UT, 2) k_tconv_fwd(const float* __restrict__ in, int ci_n, float* __restrict__ out, long long out_bs,

@@ -23,6 +23,7 @@
 #include "../../include/clamp.h"
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
+#include "packed.cuh"
 
 #include <cuda_bf16.h>
 
@@ -30,24 +31,6 @@
 
 namespace clamp {
 namespace unet_cc {
-
-typedef unsigned long long f2;   // two packed FP32
-
-__device__ __forceinline__ f2 pack2(float lo, float hi) {
-  f2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(f2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
-  f2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
 
 // BF16 mode: an operand rounded to bfloat16 (round to nearest even) and widened back.
 template <bool BF>

@@ -36,6 +36,7 @@
 #include "../../include/clamp.h"
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
+#include "packed.cuh"
 #include "tc_core.cuh"
 
 #include <cuda_bf16.h>
@@ -63,15 +64,6 @@ struct UtCfg {
   static_assert(ZT >= 1 && TX * COUT * ZT == 256, "TMEM");
   static_assert(2 * (SMEM + 1024) <= 228 * 1024, "two CTAs per SM");
 };
-
-__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
-  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
-         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
-}
-
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_addr(smem_dst)), "l"(gsrc) : "memory");
-}
 
 // wpk[((c * 27 + tap) * 2 + cg) * C_out + co] = BF16 W[co][16 c + 8 cg + k][tap], k = 0..7.
 __global__ void k_pack_weights(const float* __restrict__ W, int ci_n, int co_n, uint4* __restrict__ wpk) {

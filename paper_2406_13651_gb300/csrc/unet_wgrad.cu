@@ -33,6 +33,7 @@
 #include "../../include/clamp.h"
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
+#include "packed.cuh"
 #include "tc_core.cuh"
 
 #include <cuda_bf16.h>
@@ -44,11 +45,6 @@ namespace unet_wg {
 
 constexpr int WT = 256;   // threads per CTA
 constexpr uint32_t kWaitLimit = 1u << 22;
-
-__device__ __forceinline__ uint32_t bf16x2(float a, float b) {
-  return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a)) |
-         ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(b)) << 16);
-}
 
 // CO: output channels per CTA (16 or 32); NCG: groups of 8 input channels per CTA (1 or 2).
 template <int CO, int NCG>
