@@ -69,10 +69,10 @@ __global__ void k_flip(const float* __restrict__ W, float* __restrict__ Wf, int 
 // chains per lane in registers.  The x taps come from a window that slides along the row,
 // so four voxels cost six 16-byte shared loads and 56 FMAs, where a thread per chain paid
 // two loads per FMA (16 -> 16 at 24 x 64x64x32: 12.3 -> 1.46 ms).  Producer warps stage the next
-// chunk meanwhile (two buffers where they fit).  Bound by shared memory's return path (24 floats
-// per lane for 56 FMAs, one float per lane and clock for the four schedulers together) at one consumer
-// warp per scheduler: FMA pipe 47 % busy.  Two chains to an FFMA2 on rows staged in pairs returns
-// the same bytes and was no faster.
+// chunk meanwhile (two buffers where they fit).  Bound by the one consumer warp per scheduler: of its
+// instructions per four voxels 56 are FMAs, and it waits for six 16-byte loads (32 -> 16 at 24 x 32^3: FMA
+// pipe 42 % busy, issue slots 72 %, shared memory 0.42 wavefronts a clock).  Two chains to an FFMA2 on
+// rows staged in pairs was no faster (1.46 -> 1.45 to 1.78 ms).
 constexpr int WG_CO = 16, WG_ROWS = 4, WG_NT = 512;
 __host__ __device__ constexpr int wg_pitch(int nx) { return (nx + 3) / 4 * 4 + 8; }   // 4 zeros left, >= 4 right
 __host__ __device__ constexpr int wg_gstride(int nx) { return (WG_ROWS * ((nx + 3) / 4 * 4) + 31) / 32 * 32 + 4; }

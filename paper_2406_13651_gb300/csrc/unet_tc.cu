@@ -32,7 +32,8 @@
 // per 16 -> 16 conv at 256x256x128) and the FP32 planes' traffic (0.16 ms); measured there, mean of
 // two 16 -> 16 and one 32 -> 16: 0.69 ms with the MMAs issued by a staging thread, now 0.56 (32 -> 32 at
 // half size 0.23 -> 0.20).  What is left is the latency of a plane's round (load, store, barrier,
-// MMAs) at two CTAs per SM, which registers and shared memory allow.
+// MMAs) at two CTAs per SM, which registers and shared memory allow (16 -> 16 at 128x128x64: tensor pipe 10 % busy,
+// issue slots 39 %, DRAM 1.3 TB/s).
 #include "../../include/clamp.h"
 #include "clamp_internal.cuh"
 #include "clamp_kernels.cuh"
